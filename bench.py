@@ -100,8 +100,8 @@ def kernel_models(N, n, L, nnz, nent, S, nrhs, e, touched=None, projected=None):
     return m
 
 
-FFT_SOURCES = ("fft.cu", "common.h", "ff.h", "fft_policy.h", "fft4.cuh", "fft4_launch.cuh", "fft4_p32.cu",
-               "fft4_p64.cu", "fft4_pff.cu")
+FFT_SOURCES = ("fft.cu", "common.h", "ff.h", "fft_policy.h", "fft4.cuh", "fft4_decl.h", "fft4_launch.cuh",
+               "fft4_p32.cu", "fft4_p64.cu", "fft4_pff.cu")
 KERNEL_SOURCES = {
     "proj_gather": ("matvec.cu", "common.h", "ff.h"),
     "interp_near": ("matvec.cu", "common.h", "ff.h"),

@@ -320,17 +320,14 @@ int aim_probe_fma_peak(int which, double* tflops);
  * that order) runs one of:
  *   AIM_FFT_AUTO            the built-in rule (default): four-step;
  *   AIM_FFT_STOCKHAM        mixed-radix Stockham kernel (any 2,3,5-smooth length);
- *   AIM_FFT_FOURSTEP        four-step register kernel (compiled lengths; any
- *                           other length falls back to the Stockham kernel);
- *   AIM_FFT_FOURSTEP_SMALL  four-step with blocks of at most 128 threads
- *                           (the x pass; elsewhere as AIM_FFT_FOURSTEP);
- *   AIM_FFT_FOURSTEP_WARP   four-step x pass whose pencils go through the
- *                           three steps in groups of 1-8 warps, each group
- *                           with its own barrier (the x pass; elsewhere as
+ *   AIM_FFT_FOURSTEP        four-step register kernel (every padded length up to
+ *                           900 and 1296; a longer one falls back to the
+ *                           Stockham kernel);
+ *   AIM_FFT_FOURSTEP_SMALL  four-step with blocks of at most 128 threads, one
+ *                           pencil per thread (the x pass; elsewhere as
  *                           AIM_FFT_FOURSTEP);
- *   AIM_FFT_FOURSTEP_WIDE   four-step strided pass with twice the columns per
- *                           block (the z and y passes; on the x pass as
- *                           AIM_FFT_FOURSTEP).
+ *   AIM_FFT_FOURSTEP_WARP, AIM_FFT_FOURSTEP_WIDE  accepted; run as
+ *                           AIM_FFT_FOURSTEP.
  * aim_fft_config sets (set != NULL, [5]) and/or reads (get != NULL, [5]) the
  * choices of one precision; get receives them with AUTO resolved by the rule.
  */

@@ -16,8 +16,10 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libaim.so")
 LIB_CHECK = os.path.join(HERE, "libaim_check.so")
-SOURCES = ["api.cu", "setup.cu", "setup_dev.cu", "fft.cu", "matvec.cu", "krylov.cu", "rcs.cu", "rcs_ref.cu", "probe.cu", "profile.cu", "noalloc.cu", "autotune.cu", "nearfill.cu", "pack.cu", "fft4_p32.cu",
-           "fft4_p64.cu", "fft4_pff.cu"]
+SOURCES = ["api.cu", "setup.cu", "setup_dev.cu", "fft.cu", "matvec.cu", "krylov.cu", "rcs.cu", "rcs_ref.cu", "probe.cu", "profile.cu", "noalloc.cu", "autotune.cu", "nearfill.cu", "pack.cu"]
+# four-step FFT kernels: one object per arithmetic policy and list of lengths (AIM_FFT4_PART)
+FFT4_SOURCES = ["fft4_pff.cu", "fft4_p64.cu", "fft4_p32.cu"]
+FFT4_PARTS = 6
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = [
     "-O3",
@@ -56,12 +58,15 @@ def build(verbose=False, force=False, check=False):
     headers.append(os.path.join(os.path.dirname(HERE), "include", "aim.h"))
     objs = []
     jobs = []
-    for src in SOURCES:
+    units = [(src, src.replace(".cu", f"_{part}.o"), [f"-DAIM_FFT4_PART={part}"])
+             for part in reversed(range(FFT4_PARTS)) for src in FFT4_SOURCES]  # the longest to compile first
+    units += [(src, src.replace(".cu", ".o"), []) for src in SOURCES]
+    for src, obj, defs in units:
         s = os.path.join(CSRC, src)
-        o = os.path.join(out_dir, src.replace(".cu", ".o"))
+        o = os.path.join(out_dir, obj)
         objs.append(o)
         if force or _newer([s] + headers, o):
-            jobs.append([nvcc(), *ARCH, *flags, "-c", s, "-o", o])
+            jobs.append([nvcc(), *ARCH, *flags, *defs, "-c", s, "-o", o])
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)

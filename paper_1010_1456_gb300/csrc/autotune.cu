@@ -77,9 +77,8 @@ static int autotune(aim_ctx* c, int precision, int nrhs, int reps, int32_t* kern
     int best = AIM_FFT_AUTO;
     double best_ms = 0.0;
     for (int k = AIM_FFT_STOCKHAM; k < AIM_FFT_KERNELS && rc == AIM_OK; ++k) {
-      // the x pass has the block-size and warp-group variants, the strided passes the wide one
-      const bool x_only = k == AIM_FFT_FOURSTEP_SMALL || k == AIM_FFT_FOURSTEP_WARP;
-      if (pass == 2 ? k == AIM_FFT_FOURSTEP_WIDE : x_only) continue;
+      // the x pass has a small-block variant; the warp-group and wide choices run the plain four-step kernel
+      if (k == AIM_FFT_FOURSTEP_WARP || k == AIM_FFT_FOURSTEP_WIDE || (k == AIM_FFT_FOURSTEP_SMALL && pass != 2)) continue;
       c->fft_kernel[pol][pass] = k;
       double ms = 0.0;
       rc = time_pass(c, pass, x, y, nrhs, precision, reps, &ms);

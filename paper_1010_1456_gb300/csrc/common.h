@@ -137,8 +137,8 @@ template <typename R> struct PrecData {
 // Float-float copies of the AIM_C128 path: spectrum, twiddles and grids of
 // the FFT passes, and (rounded once from the FP64 setup arrays) the weights
 // and near entries of the projection and interpolation.  A float-float real
-// is (hi, lo) with value hi + lo; a complex one is float4 (re.hi, re.lo,
-// im.hi, im.lo).
+// is (hi, lo) with value hi + lo; a complex one is float4 (re.hi, im.hi,
+// re.lo, im.lo).
 struct FFData {
   float4* ghat = nullptr;
   float4* tw[3] = {nullptr, nullptr, nullptr};

@@ -23,7 +23,7 @@
 //
 // The butterflies are written once over an arithmetic policy:
 //   P32 complex64 (float2), P64 complex128 (double2) and PFF complex
-//   float-float (float4 = re.hi, re.lo, im.hi, im.lo; about 48 bits, on the
+//   float-float (float4 = re.hi, im.hi, re.lo, im.lo; about 48 bits, on the
 //   FP32 pipes; see ff.h).  Per-stage index arithmetic uses precomputed
 //   multiply-shift division, so no integer division runs in the kernels.
 #include <cmath>
@@ -33,6 +33,7 @@
 #include "common.h"
 #include "ff.h"
 #include "fft4.cuh"
+#include "fft4_decl.h"
 #include "fft_policy.h"
 #include "geom.h"
 
@@ -161,30 +162,75 @@ __device__ typename P::S* stockham(typename P::S* b0, typename P::S* b1, const F
 // ------------------------------------------------------------------ strided pass
 using StridedArgs = StridedArgs4;
 
-// Four-step kernels per policy (fft4_p32.cu, fft4_p64.cu, fft4_pff.cu):
-// 1 launched, 0 no kernel for this length, < 0 minus an error code.
-int fft4_strided_p32(aim_ctx*, const char*, bool, const float2*, float2*, const StridedArgs4&, int, int,
-                     const float2*, bool);
-int fft4_strided_p64(aim_ctx*, const char*, bool, const double2*, double2*, const StridedArgs4&, int, int,
-                     const double2*, bool);
-int fft4_strided_pff(aim_ctx*, const char*, bool, const float4*, float4*, const StridedArgs4&, int, int,
-                     const float4*, bool);
-int fft4_x_p32(aim_ctx*, const char*, float2*, const XArgs4&, int, const float2*, const float2*, int, bool);
-int fft4_x_p64(aim_ctx*, const char*, double2*, const XArgs4&, int, const double2*, const double2*, int, bool);
-int fft4_x_pff(aim_ctx*, const char*, float4*, const XArgs4&, int, const float4*, const float4*, int, bool);
+// Four-step kernels per policy (fft4_decl.h), by the list that holds length L.
 template <class P> struct Fft4;
 template <> struct Fft4<P32> {
-  template <class... A> static int strided(A... a) { return fft4_strided_p32(a...); }
-  template <class... A> static int x(A... a) { return fft4_x_p32(a...); }
+  template <class... A> static int strided(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_strided_p32<0>(a...);
+      case 1: return fft4_strided_p32<1>(a...);
+      case 2: return fft4_strided_p32<2>(a...);
+      case 3: return fft4_strided_p32<3>(a...);
+      case 4: return fft4_strided_p32<4>(a...);
+      default: return fft4_strided_p32<5>(a...);
+    }
+  }
+  template <class... A> static int x(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_x_p32<0>(a...);
+      case 1: return fft4_x_p32<1>(a...);
+      case 2: return fft4_x_p32<2>(a...);
+      case 3: return fft4_x_p32<3>(a...);
+      case 4: return fft4_x_p32<4>(a...);
+      default: return fft4_x_p32<5>(a...);
+    }
+  }
 };
 template <> struct Fft4<P64> {
-  template <class... A> static int strided(A... a) { return fft4_strided_p64(a...); }
-  template <class... A> static int x(A... a) { return fft4_x_p64(a...); }
+  template <class... A> static int strided(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_strided_p64<0>(a...);
+      case 1: return fft4_strided_p64<1>(a...);
+      case 2: return fft4_strided_p64<2>(a...);
+      case 3: return fft4_strided_p64<3>(a...);
+      case 4: return fft4_strided_p64<4>(a...);
+      default: return fft4_strided_p64<5>(a...);
+    }
+  }
+  template <class... A> static int x(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_x_p64<0>(a...);
+      case 1: return fft4_x_p64<1>(a...);
+      case 2: return fft4_x_p64<2>(a...);
+      case 3: return fft4_x_p64<3>(a...);
+      case 4: return fft4_x_p64<4>(a...);
+      default: return fft4_x_p64<5>(a...);
+    }
+  }
 };
 template <> struct Fft4<PFF> {
-  template <class... A> static int strided(A... a) { return fft4_strided_pff(a...); }
-  template <class... A> static int x(A... a) { return fft4_x_pff(a...); }
+  template <class... A> static int strided(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_strided_pff<0>(a...);
+      case 1: return fft4_strided_pff<1>(a...);
+      case 2: return fft4_strided_pff<2>(a...);
+      case 3: return fft4_strided_pff<3>(a...);
+      case 4: return fft4_strided_pff<4>(a...);
+      default: return fft4_strided_pff<5>(a...);
+    }
+  }
+  template <class... A> static int x(int L, A... a) {
+    switch (fourstep_part(L)) {
+      case 0: return fft4_x_pff<0>(a...);
+      case 1: return fft4_x_pff<1>(a...);
+      case 2: return fft4_x_pff<2>(a...);
+      case 3: return fft4_x_pff<3>(a...);
+      case 4: return fft4_x_pff<4>(a...);
+      default: return fft4_x_pff<5>(a...);
+    }
+  }
 };
+static_assert(kFourStepParts == 6, "one case per list above");
 
 // Output element conversion of a pass (identity for every policy in use).
 template <class S, class O> struct OutConv {
@@ -342,7 +388,7 @@ static int strided_pass(aim_ctx* c, int pass, const char* name, const typename P
                         const StridedArgs& a, int G, const FftPlan* plan_dev, int L, const typename P::S* tw) {
   const int k = fft_kernel_for(c, policy_index<P>(), pass);
   if (k != AIM_FFT_STOCKHAM) {
-    const int rc = Fft4<P>::strided(c, name, INV, in, out, a, G, L, tw, k == AIM_FFT_FOURSTEP_WIDE);
+    const int rc = Fft4<P>::strided(L, c, name, INV, in, out, a, G, L, tw);
     if (rc == 1) return AIM_OK;
     if (rc < 0) return -rc;
   }
@@ -356,8 +402,7 @@ static int x_pass(aim_ctx* c, const char* name, typename P::S* buf, XArgs a, con
   if (k != AIM_FFT_STOCKHAM) {
     XArgs4 x4{};
     x4.nx = a.nx; x4.Ly = a.rows_y; x4.Lz = a.rows_z; x4.G = a.G; x4.sG = a.sG; x4.hx = a.hx; x4.hy = a.hy;
-    const int rc = Fft4<P>::x(c, name, buf, x4, L, ghat, tw, k == AIM_FFT_FOURSTEP_SMALL ? 128 : 256,
-                              k == AIM_FFT_FOURSTEP_WARP);
+    const int rc = Fft4<P>::x(L, c, name, buf, x4, L, ghat, tw, k == AIM_FFT_FOURSTEP_SMALL ? 128 : 256);
     if (rc == 1) return AIM_OK;
     if (rc < 0) return -rc;
   }
@@ -464,7 +509,7 @@ __global__ void extract_octant(const double2* full, double2* oct64, float2* oct3
     oct64[e] = v;
     oct32[e] = make_float2((float)v.x, (float)v.y);
     const ff re = ff_from_double(v.x), im = ff_from_double(v.y);
-    octff[e] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    octff[e] = make_float4(re.hi, im.hi, re.lo, im.lo);
   }
 }
 
@@ -485,7 +530,7 @@ int build_ghat(aim_ctx* c) {
   s.sG_out = total; s.sA_out = Lx; s.sP_out = (long long)Ly * Lx;
   // full transforms; four-step kernels where the length has one (longer than the Stockham kernel allows)
   const auto pass = [&](const char* name, const double2* in, double2* out, const StridedArgs& sa, int d) -> int {
-    const int rc = Fft4<P64>::strided(c, name, false, in, out, sa, 1, c->L[d], c->p64.tw[d], false);
+    const int rc = Fft4<P64>::strided(c->L[d], c, name, false, in, out, sa, 1, c->L[d], c->p64.tw[d]);
     if (rc == 1) return AIM_OK;
     if (rc < 0) return -rc;
     return launch_strided<P64, false>(c, name, in, out, sa, 1, c->plan_dev + d, c->L[d], c->p64.tw[d]);

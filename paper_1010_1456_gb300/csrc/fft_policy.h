@@ -2,7 +2,7 @@
 // DFTs.
 //
 // Policies: P32 complex64 (float2), P64 complex128 (double2), PFF complex
-// float-float (float4 = re.hi, re.lo, im.hi, im.lo; about 48 bits on the FP32
+// float-float (float4 = re.hi, im.hi, re.lo, im.lo; about 48 bits on the FP32
 // pipes, see ff.h).  Every butterfly is written once over a policy.
 //
 // RegDFT<P, N, INV>::run(v) transforms N values held in registers (natural
@@ -85,26 +85,33 @@ struct P32 {
   using S = float2;  // storage
   using T = float2;  // work
   static constexpr int kTX = 16;
-  AIM_HD static T ld(const S& s) { return s; }
-  AIM_HD static S st(const T& t) { return t; }
-  AIM_HD static T zero() { return make_float2(0.f, 0.f); }
-  AIM_HD static T add(T a, T b) { return make_float2(a.x + b.x, a.y + b.y); }
-  AIM_HD static T sub(T a, T b) { return make_float2(a.x - b.x, a.y - b.y); }
-  AIM_HD static T neg(T a) { return make_float2(-a.x, -a.y); }
-  AIM_HD static T mul(T a, T b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-  AIM_HD static T mulr(T a, double, float c, float) { return make_float2(a.x * c, a.y * c); }
+  __device__ static T ld(const S& s) { return s; }
+  __device__ static S st(const T& t) { return t; }
+  __device__ static T zero() { return make_float2(0.f, 0.f); }
+  __device__ static T add(T a, T b) { return add2(a, b); }
+  __device__ static T sub(T a, T b) { return sub2(a, b); }
+  __device__ static T neg(T a) { return neg2(a); }
+  __device__ static T mul(T a, T b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+  __device__ static T mulr(T a, double, float c, float) { return mul2(a, both(c)); }
+  __device__ static T madr(T m, T a, double, float c, float) { return fma2(a, both(c), m); }  // m + c a
+  __device__ static T sub_half(T m, T a) { return fma2(a, both(-0.5f), m); }                  // m - a / 2
+  __device__ static T neg_half(T a) { return mul2(a, both(-0.5f)); }
   // a * (c + i s) for compile-time constants
-  AIM_HD static T mulc(T a, double, float c, float, double, float s, float) {
-    return make_float2(a.x * c - a.y * s, a.x * s + a.y * c);
+  __device__ static T mulc(T a, double, float c, float, double, float s, float) {
+    return fma2(swap2(a), make_float2(-s, s), mul2(a, both(c)));
   }
-  AIM_HD static T half(T a) { return make_float2(0.5f * a.x, 0.5f * a.y); }
-  template <bool INV> AIM_HD static T mul_mi(T a) { return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x); }
-  // m + sg * mul_mi(c d) with one fused multiply-add per component (sg = +-1)
-  template <bool INV, int SG> AIM_HD static T add_mi_scaled(T m, T d, double, float c, float) {
+  template <bool INV> __device__ static T mul_mi(T a) {
+    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+  }
+  // m + sg * mul_mi(c d) and m + sg * mul_mi(d) (sg = +-1)
+  template <bool INV, int SG> __device__ static T add_mi_scaled(T m, T d, double, float c, float) {
     const float cs = SG * (INV ? -c : c);
-    return make_float2(fmaf(cs, d.y, m.x), fmaf(-cs, d.x, m.y));
+    return fma2(swap2(d), make_float2(cs, -cs), m);
   }
-  AIM_HD static T conj_if(T w, bool c) { return c ? make_float2(w.x, -w.y) : w; }
+  template <bool INV, int SG> __device__ static T add_mi(T m, T d) {
+    return add_mi_scaled<INV, SG>(m, d, 1.0, 1.f, 0.f);
+  }
+  __device__ static T conj_if(T w, bool c) { return c ? make_float2(w.x, -w.y) : w; }
 };
 
 struct P64 {
@@ -119,91 +126,160 @@ struct P64 {
   AIM_HD static T neg(T a) { return make_double2(-a.x, -a.y); }
   AIM_HD static T mul(T a, T b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
   AIM_HD static T mulr(T a, double c, float, float) { return make_double2(a.x * c, a.y * c); }
+  AIM_HD static T madr(T m, T a, double c, float, float) { return make_double2(fma(c, a.x, m.x), fma(c, a.y, m.y)); }
+  AIM_HD static T sub_half(T m, T a) { return make_double2(fma(-0.5, a.x, m.x), fma(-0.5, a.y, m.y)); }
+  AIM_HD static T neg_half(T a) { return make_double2(-0.5 * a.x, -0.5 * a.y); }
   AIM_HD static T mulc(T a, double c, float, float, double s, float, float) {
     return make_double2(a.x * c - a.y * s, a.x * s + a.y * c);
   }
-  AIM_HD static T half(T a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
   template <bool INV> AIM_HD static T mul_mi(T a) { return INV ? make_double2(-a.y, a.x) : make_double2(a.y, -a.x); }
   template <bool INV, int SG> AIM_HD static T add_mi_scaled(T m, T d, double c, float, float) {
     const double cs = SG * (INV ? -c : c);
     return make_double2(fma(cs, d.y, m.x), fma(-cs, d.x, m.y));
   }
+  template <bool INV, int SG> AIM_HD static T add_mi(T m, T d) {
+    const T t = mul_mi<INV>(d);
+    return SG > 0 ? add(m, t) : sub(m, t);
+  }
   AIM_HD static T conj_if(T w, bool c) { return c ? make_double2(w.x, -w.y) : w; }
 };
 
 struct PFF {
-  using S = float4;
-  using T = cff;
+  using S = float4;  // (re.hi, im.hi, re.lo, im.lo)
+  using T = cff2;
   static constexpr int kTX = 8;
-  __device__ static T ld(const S& s) { return cff{ff{s.x, s.y}, ff{s.z, s.w}}; }
-  __device__ static S st(const T& t) { return make_float4(t.re.hi, t.re.lo, t.im.hi, t.im.lo); }
-  __device__ static T zero() { return cff{ff{0.f, 0.f}, ff{0.f, 0.f}}; }
-  __device__ static T add(T a, T b) { return cff{ff_add_lazy(a.re, b.re), ff_add_lazy(a.im, b.im)}; }
-  __device__ static T sub(T a, T b) { return cff{ff_sub_lazy(a.re, b.re), ff_sub_lazy(a.im, b.im)}; }
-  __device__ static T neg(T a) { return cff{ff_neg(a.re), ff_neg(a.im)}; }
-  __device__ static T mul(T a, T b) {
-    return cff{ff_dot2(a.re, b.re, ff_neg(a.im), b.im), ff_dot2(a.re, b.im, a.im, b.re)};
-  }
+  __device__ static T ld(const S& s) { return cff2_ld(s); }
+  __device__ static S st(const T& t) { return cff2_st(t); }
+  __device__ static T zero() { return cff2_zero(); }
+  // additions without the closing renormalisation: every value feeds further arithmetic
+  __device__ static T add(T a, T b) { return cff2_add_lazy(a, b); }
+  __device__ static T sub(T a, T b) { return cff2_add_lazy(a, cff2_neg(b)); }
+  __device__ static T neg(T a) { return cff2_neg(a); }
+  __device__ static T mul(T a, T b) { return cff2_dot2(cff2_re(a), b, cff2_im(a), cff2_times_i(b)); }
   __device__ static T mulr(T a, double, float ch, float cl) {
-    const ff c{ch, cl};
-    return cff{ff_mul(a.re, c), ff_mul(a.im, c)};
+    const float2 h = both(ch), p = mul2(a.hi, h);
+    float2 e = fma2(a.hi, h, neg2(p));
+    e = fma2(a.hi, both(cl), e);
+    e = fma2(a.lo, h, e);
+    return fast_two_sum2(p, e);
   }
+  __device__ static T madr(T m, T a, double c, float ch, float cl) { return add(m, mulr(a, c, ch, cl)); }
+  __device__ static T neg_half(T a) { return cff2{mul2(a.hi, both(-0.5f)), mul2(a.lo, both(-0.5f))}; }
+  __device__ static T sub_half(T m, T a) { return add(m, neg_half(a)); }
   __device__ static T mulc(T a, double, float ch, float cl, double, float sh, float sl) {
-    const ff c{ch, cl}, s{sh, sl};
-    return cff{ff_dot2(a.re, c, ff_neg(a.im), s), ff_dot2(a.re, s, a.im, c)};
+    return cff2_dot2(a, cff2{both(ch), both(cl)}, cff2{swap2(a.hi), swap2(a.lo)},
+                     cff2{make_float2(-sh, sh), make_float2(-sl, sl)});
   }
-  __device__ static T half(T a) { return cff{ff{0.5f * a.re.hi, 0.5f * a.re.lo}, ff{0.5f * a.im.hi, 0.5f * a.im.lo}}; }
-  template <bool INV> __device__ static T mul_mi(T a) { return INV ? cff{ff_neg(a.im), a.re} : cff{a.im, ff_neg(a.re)}; }
+  template <bool INV> __device__ static T mul_mi(T a) { return INV ? cff2_times_i(a) : cff2_neg(cff2_times_i(a)); }
   template <bool INV, int SG> __device__ static T add_mi_scaled(T m, T d, double c, float ch, float cl) {
-    const T t = mul_mi<INV>(mulr(d, c, ch, cl));
-    return SG > 0 ? add(m, t) : sub(m, t);
+    return add_mi<INV, SG>(m, mulr(d, c, ch, cl));
   }
-  __device__ static T conj_if(T w, bool c) { return c ? cff{w.re, ff_neg(w.im)} : w; }
+  template <bool INV, int SG> __device__ static T add_mi(T m, T d) {
+    const T t = mul_mi<(SG > 0) == INV>(d);
+    return add(m, t);
+  }
+  __device__ static T conj_if(T w, bool c) {
+    return c ? cff2{make_float2(w.hi.x, -w.hi.y), make_float2(w.lo.x, -w.lo.y)} : w;
+  }
 };
 
 // Real constants as (double value, float hi, float lo).
 #define AIM_RC(c) (c), (float)(c), (float)((c) - (double)(float)(c))
 
 // ------------------------------------------------------------------ small butterflies
-template <class P, bool INV> AIM_HD __forceinline__ void dft2(typename P::T* v) {
+// Each takes a mask Z of the inputs that are not known to be zero (bit i:
+// v[i]); the others are neither read nor added.  A zero-padded transform
+// whose upper half is zero drops the additions of its first stage this way.
+template <class P, bool A, bool B> AIM_HD __forceinline__ typename P::T add_z(typename P::T a, typename P::T b) {
+  if constexpr (A && B) return P::add(a, b);
+  else if constexpr (A) return a;
+  else if constexpr (B) return b;
+  else return P::zero();
+}
+template <class P, bool A, bool B> AIM_HD __forceinline__ typename P::T sub_z(typename P::T a, typename P::T b) {
+  if constexpr (A && B) return P::sub(a, b);
+  else if constexpr (A) return a;
+  else if constexpr (B) return P::neg(b);
+  else return P::zero();
+}
+// m + sg * mul_mi(d)
+template <class P, bool INV, int SG, bool M, bool D>
+AIM_HD __forceinline__ typename P::T add_mi_z(typename P::T m, typename P::T d) {
+  if constexpr (M && D) return P::template add_mi<INV, SG>(m, d);
+  else if constexpr (M) return m;
+  else if constexpr (D) return P::template mul_mi<(SG > 0) == INV>(d);
+  else return P::zero();
+}
+constexpr bool has(unsigned long long z, int i) { return (z >> i) & 1; }
+constexpr unsigned long long all_mask(int n) { return n >= 64 ? ~0ull : (1ull << n) - 1; }
+
+template <class P, bool INV, unsigned long long Z = 3> AIM_HD __forceinline__ void dft2(typename P::T* v) {
   const typename P::T a = v[0], b = v[1];
-  v[0] = P::add(a, b);
-  v[1] = P::sub(a, b);
+  v[0] = add_z<P, has(Z, 0), has(Z, 1)>(a, b);
+  v[1] = sub_z<P, has(Z, 0), has(Z, 1)>(a, b);
 }
-template <class P, bool INV> AIM_HD __forceinline__ void dft3(typename P::T* v) {
+template <class P, bool INV, unsigned long long Z = 7> AIM_HD __forceinline__ void dft3(typename P::T* v) {
   using T = typename P::T;
-  const T a = v[0], s = P::add(v[1], v[2]), d = P::sub(v[1], v[2]);
-  const T m = P::sub(a, P::half(s));
-  // v1, v2 = m +- (-i) sin(2 pi / 3) d (forward; +i inverse), each a fused multiply-add
-  v[0] = P::add(a, s);
-  v[1] = P::template add_mi_scaled<INV, 1>(m, d, AIM_RC(0.86602540378443864676));
-  v[2] = P::template add_mi_scaled<INV, -1>(m, d, AIM_RC(0.86602540378443864676));
+  constexpr bool z0 = has(Z, 0), z1 = has(Z, 1), z2 = has(Z, 2), zs = z1 || z2;
+  const T a = v[0], s = add_z<P, z1, z2>(v[1], v[2]), d = sub_z<P, z1, z2>(v[1], v[2]);
+  v[0] = add_z<P, z0, zs>(a, s);
+  if constexpr (zs) {
+    T m;
+    if constexpr (z0) m = P::sub_half(a, s);
+    else m = P::neg_half(s);
+    // v1, v2 = m +- (-i) sin(2 pi / 3) d (forward; +i inverse), each a fused multiply-add
+    v[1] = P::template add_mi_scaled<INV, 1>(m, d, AIM_RC(0.86602540378443864676));
+    v[2] = P::template add_mi_scaled<INV, -1>(m, d, AIM_RC(0.86602540378443864676));
+  } else {
+    v[1] = v[2] = a;
+  }
 }
-template <class P, bool INV> AIM_HD __forceinline__ void dft4(typename P::T* v) {
+template <class P, bool INV, unsigned long long Z = 15> AIM_HD __forceinline__ void dft4(typename P::T* v) {
   using T = typename P::T;
-  const T s02 = P::add(v[0], v[2]), d02 = P::sub(v[0], v[2]);
-  const T s13 = P::add(v[1], v[3]), d13 = P::template mul_mi<INV>(P::sub(v[1], v[3]));
-  v[0] = P::add(s02, s13);
-  v[2] = P::sub(s02, s13);
-  v[1] = P::add(d02, d13);
-  v[3] = P::sub(d02, d13);
+  constexpr bool z0 = has(Z, 0), z1 = has(Z, 1), z2 = has(Z, 2), z3 = has(Z, 3), ze = z0 || z2, zo = z1 || z3;
+  const T s02 = add_z<P, z0, z2>(v[0], v[2]), d02 = sub_z<P, z0, z2>(v[0], v[2]);
+  const T s13 = add_z<P, z1, z3>(v[1], v[3]), d13 = sub_z<P, z1, z3>(v[1], v[3]);
+  v[0] = add_z<P, ze, zo>(s02, s13);
+  v[2] = sub_z<P, ze, zo>(s02, s13);
+  v[1] = add_mi_z<P, INV, 1, ze, zo>(d02, d13);
+  v[3] = add_mi_z<P, INV, -1, ze, zo>(d02, d13);
 }
-template <class P, bool INV> AIM_HD __forceinline__ void dft5(typename P::T* v) {
+template <class P, bool INV, unsigned long long Z = 31> AIM_HD __forceinline__ void dft5(typename P::T* v) {
   using T = typename P::T;
+  constexpr bool z0 = has(Z, 0), z1 = has(Z, 1), z2 = has(Z, 2), z3 = has(Z, 3), z4 = has(Z, 4);
+  constexpr bool za = z1 || z4, zb = z2 || z3;
   const T a0 = v[0];
-  const T t1 = P::add(v[1], v[4]), t2 = P::add(v[2], v[3]);
-  const T t3 = P::sub(v[1], v[4]), t4 = P::sub(v[2], v[3]);
+  if constexpr (!za && !zb) {
+    v[1] = v[2] = v[3] = v[4] = a0;
+    return;
+  }
+  const T t1 = add_z<P, z1, z4>(v[1], v[4]), t2 = add_z<P, z2, z3>(v[2], v[3]);
+  const T t3 = sub_z<P, z1, z4>(v[1], v[4]), t4 = sub_z<P, z2, z3>(v[2], v[3]);
   // cos(2pi/5), cos(4pi/5), sin(2pi/5), sin(4pi/5)
-  const T b1 = P::add(a0, P::add(P::mulr(t1, AIM_RC(0.30901699437494742410)), P::mulr(t2, AIM_RC(-0.80901699437494742410))));
-  const T b2 = P::add(a0, P::add(P::mulr(t1, AIM_RC(-0.80901699437494742410)), P::mulr(t2, AIM_RC(0.30901699437494742410))));
-  const T u1 = P::add(P::mulr(t3, AIM_RC(0.95105651629515357212)), P::mulr(t4, AIM_RC(0.58778525229247312917)));
-  const T u2 = P::sub(P::mulr(t3, AIM_RC(0.58778525229247312917)), P::mulr(t4, AIM_RC(0.95105651629515357212)));
-  const T e1 = P::template mul_mi<INV>(u1), e2 = P::template mul_mi<INV>(u2);
-  v[0] = P::add(a0, P::add(t1, t2));
-  v[1] = P::add(b1, e1);
-  v[4] = P::sub(b1, e1);
-  v[2] = P::add(b2, e2);
-  v[3] = P::sub(b2, e2);
+  T b1, b2, u1, u2;
+  if constexpr (za && zb) {
+    b1 = P::madr(P::mulr(t1, AIM_RC(0.30901699437494742410)), t2, AIM_RC(-0.80901699437494742410));
+    b2 = P::madr(P::mulr(t1, AIM_RC(-0.80901699437494742410)), t2, AIM_RC(0.30901699437494742410));
+    u1 = P::madr(P::mulr(t3, AIM_RC(0.95105651629515357212)), t4, AIM_RC(0.58778525229247312917));
+    u2 = P::madr(P::mulr(t3, AIM_RC(0.58778525229247312917)), t4, AIM_RC(-0.95105651629515357212));
+  } else if constexpr (za) {
+    b1 = P::mulr(t1, AIM_RC(0.30901699437494742410));
+    b2 = P::mulr(t1, AIM_RC(-0.80901699437494742410));
+    u1 = P::mulr(t3, AIM_RC(0.95105651629515357212));
+    u2 = P::mulr(t3, AIM_RC(0.58778525229247312917));
+  } else {
+    b1 = P::mulr(t2, AIM_RC(-0.80901699437494742410));
+    b2 = P::mulr(t2, AIM_RC(0.30901699437494742410));
+    u1 = P::mulr(t4, AIM_RC(0.58778525229247312917));
+    u2 = P::mulr(t4, AIM_RC(-0.95105651629515357212));
+  }
+  b1 = add_z<P, z0, true>(a0, b1);
+  b2 = add_z<P, z0, true>(a0, b2);
+  v[0] = add_z<P, z0, true>(a0, add_z<P, za, zb>(t1, t2));
+  v[1] = P::template add_mi<INV, 1>(b1, u1);
+  v[4] = P::template add_mi<INV, -1>(b1, u1);
+  v[2] = P::template add_mi<INV, 1>(b2, u2);
+  v[3] = P::template add_mi<INV, -1>(b2, u2);
 }
 
 // ------------------------------------------------------------------ register DFT
@@ -245,18 +321,34 @@ template <class P, int N, int E, bool INV> AIM_HD __forceinline__ typename P::T 
   }
 }
 
-template <class P, int N, bool INV> struct RegDFT {
+// The mask of the inputs first, first + step, ... (count of them, mod n) of a DFT of length n
+constexpr unsigned long long sub_mask(unsigned long long z, int n, int first, int step, int count) {
+  unsigned long long m = 0;
+  for (int i = 0; i < count; ++i)
+    if (has(z, (first + step * i) % n)) m |= 1ull << i;
+  return m;
+}
+// Bit j: whether the sub-transform j (inputs base j + step i mod n, i < count) has a nonzero input
+constexpr unsigned long long group_mask(unsigned long long z, int n, int groups, int base, int step, int count) {
+  unsigned long long m = 0;
+  for (int j = 0; j < groups; ++j)
+    if (sub_mask(z, n, (base * j) % n, step, count)) m |= 1ull << j;
+  return m;
+}
+
+// Z: the inputs that are not known to be zero (see the butterflies).
+template <class P, int N, bool INV, unsigned long long Z = all_mask(N)> struct RegDFT {
   using T = typename P::T;
   AIM_HD __forceinline__ static void run(T* v) {
     if constexpr (N == 1) {
     } else if constexpr (N == 2) {
-      dft2<P, INV>(v);
+      dft2<P, INV, Z>(v);
     } else if constexpr (N == 3) {
-      dft3<P, INV>(v);
+      dft3<P, INV, Z>(v);
     } else if constexpr (N == 4) {
-      dft4<P, INV>(v);
+      dft4<P, INV, Z>(v);
     } else if constexpr (N == 5) {
-      dft5<P, INV>(v);
+      dft5<P, INV, Z>(v);
     } else if constexpr (coprime_factor(N) != 0) {
       // Good-Thomas prime-factor split N = R M, gcd(R, M) = 1: input index
       // n = (M j + R i) mod N, output index k = (M a k1 + R b k2) mod N with
@@ -264,15 +356,17 @@ template <class P, int N, bool INV> struct RegDFT {
       constexpr int R = coprime_factor(N);
       constexpr int M = N / R;
       constexpr int A = inv_mod(M % R, R), B = inv_mod(R % M, M);
+      constexpr unsigned long long ZG = group_mask(Z, N, R, M, R, M);
       T sub[R][M];
       static_for<0, R>([&](auto j) {
         static_for<0, M>([&](auto i) { sub[j][i] = v[(M * decltype(j)::value + R * decltype(i)::value) % N]; });
-        RegDFT<P, M, INV>::run(sub[j]);
+        constexpr unsigned long long ZS = sub_mask(Z, N, (M * decltype(j)::value) % N, R, M);
+        if constexpr (ZS != 0) RegDFT<P, M, INV, ZS>::run(sub[j]);
       });
       static_for<0, M>([&](auto k2) {
         T t[R];
         static_for<0, R>([&](auto j) { t[j] = sub[j][k2]; });
-        RegDFT<P, R, INV>::run(t);
+        RegDFT<P, R, INV, ZG>::run(t);
         static_for<0, R>([&](auto k1) {
           v[(M * A * decltype(k1)::value + R * B * decltype(k2)::value) % N] = t[k1];
         });
@@ -281,17 +375,22 @@ template <class P, int N, bool INV> struct RegDFT {
       constexpr int R = first_factor(N);
       constexpr int M = N / R;
       static_assert(R * M == N && R > 1 && R <= 5, "register DFT length must be 2,3,5-smooth");
+      constexpr unsigned long long ZG = group_mask(Z, N, R, 1, R, M);
       T sub[R][M];
       static_for<0, R>([&](auto j) {
         static_for<0, M>([&](auto i) { sub[j][i] = v[R * i + j]; });
-        RegDFT<P, M, INV>::run(sub[j]);
+        constexpr unsigned long long ZS = sub_mask(Z, N, decltype(j)::value, R, M);
+        if constexpr (ZS != 0) RegDFT<P, M, INV, ZS>::run(sub[j]);
       });
       static_for<0, M>([&](auto k2) {
         T t[R];
         static_for<0, R>([&](auto j) {
-          t[j] = twiddle_c<P, N, decltype(j)::value * decltype(k2)::value, INV>(sub[j][k2]);
+          if constexpr (has(ZG, decltype(j)::value))
+            t[j] = twiddle_c<P, N, decltype(j)::value * decltype(k2)::value, INV>(sub[j][k2]);
+          else
+            t[j] = P::zero();
         });
-        RegDFT<P, R, INV>::run(t);
+        RegDFT<P, R, INV, ZG>::run(t);
         static_for<0, R>([&](auto q) { v[k2 + M * q] = t[q]; });
       });
     }

@@ -588,7 +588,7 @@ __global__ void k_real_to_ff(const double* __restrict__ in, float2* __restrict__
 __global__ void k_cplx_to_ff(const double2* __restrict__ in, float4* __restrict__ out, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const ff re = ff_from_double(in[i].x), im = ff_from_double(in[i].y);
-    out[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    out[i] = make_float4(re.hi, im.hi, re.lo, im.lo);
   }
 }
 // [nent][4] FP64 weights -> [nent][2] float4: high parts, then low parts.
@@ -632,26 +632,24 @@ __global__ void __launch_bounds__(256) proj_gather_ff(const float4* __restrict__
       continue;
     }
     for (int b0 = 0; b0 < nrhs; b0 += BC) {
-      ff a[BC][4][2];
+      cff2 a[BC][4];
 #pragma unroll
       for (int q = 0; q < BC; ++q)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a[q][c][0] = a[q][c][1] = ffv(0.f, 0.f);
+        for (int c = 0; c < 4; ++c) a[q][c] = cff2_zero();
       for (int e = e0 + lane; e < e1; e += 4) {
         const float4 wh = w[2 * e], wl = w[2 * e + 1];
         const float4* xc = x + mm[e];
         float4 xv[BC];
 #pragma unroll
         for (int q = 0; q < BC; ++q) xv[q] = b0 + q < nrhs ? xc[(long long)(b0 + q) * N] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const ff wc[4] = {ffv(wh.x, wl.x), ffv(wh.y, wl.y), ffv(wh.z, wl.z), ffv(wh.w, wl.w)};
+        const cff2 wc[4] = {cff2_both(ffv(wh.x, wl.x)), cff2_both(ffv(wh.y, wl.y)), cff2_both(ffv(wh.z, wl.z)),
+                            cff2_both(ffv(wh.w, wl.w))};
 #pragma unroll
         for (int q = 0; q < BC; ++q) {
-          const ff xr = ffv(xv[q].x, xv[q].y), xi = ffv(xv[q].z, xv[q].w);
+          const cff2 xq = cff2_ld(xv[q]);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            a[q][c][0] = ff_mad(wc[c], xr, a[q][c][0]);
-            a[q][c][1] = ff_mad(wc[c], xi, a[q][c][1]);
-          }
+          for (int c = 0; c < 4; ++c) a[q][c] = cff2_mad(wc[c], xq, a[q][c]);
         }
       }
 #pragma unroll
@@ -659,23 +657,14 @@ __global__ void __launch_bounds__(256) proj_gather_ff(const float4* __restrict__
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1)
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              const ff t = ffv(__shfl_xor_sync(0xffffffffu, a[q][c][r].hi, o, 4),
-                               __shfl_xor_sync(0xffffffffu, a[q][c][r].lo, o, 4));
-              a[q][c][r] = ff_add(a[q][c][r], t);
-            }
+          for (int c = 0; c < 4; ++c) a[q][c] = cff2_add(a[q][c], cff2_shfl_xor(a[q][c], o, 4));
         if (live && b0 + q < nrhs) {
           // lane c writes component c
-          ff re = a[q][0][0], im = a[q][0][1];
+          cff2 v = a[q][0];
 #pragma unroll
           for (int c = 1; c < 4; ++c)
-            if (lane == c) {
-              re = a[q][c][0];
-              im = a[q][c][1];
-            }
-          Q[(long long)(b0 + q) * 4 * Nc + (long long)lane * Nc + u] = make_float4(re.hi, re.lo, im.hi, im.lo);
+            if (lane == c) v = a[q][c];
+          Q[(long long)(b0 + q) * 4 * Nc + (long long)lane * Nc + u] = cff2_st(v);
         }
       }
     }
@@ -708,55 +697,40 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
 #else
   const int Sc = S;
 #endif
-  const ff kv = ffv(fvec.x, fvec.y), kr = ffv(frho.x, frho.y), km = ffv(fmf.x, fmf.y);
+  const cff2 kv = cff2_both(ffv(fvec.x, fvec.y)), kr = cff2_both(ffv(-frho.x, -frho.y)),
+             km = cff2_both(ffv(-fmf.x, -fmf.y));
   for (int b = 0; b < nrhs; ++b) {
     const float4* Pb = Phi + (long long)b * 4 * Nc;
-    ff avr = ffv(0.f, 0.f), avi = avr, arr = avr, ari = avr, anr = avr, ani = avr, amr = avr, ami = avr;
+    cff2 av = cff2_zero(), ar = av, an = av, am = av;
     for (int s = lane; s < Sc; s += 8) {
       const long long node = b0 + (long long)s_off[s];
-      const float4 px = Pb[node], py = Pb[Nc + node], pz = Pb[2 * Nc + node], pr = Pb[3 * Nc + node];
+      const cff2 px = cff2_ld(Pb[node]), py = cff2_ld(Pb[Nc + node]), pz = cff2_ld(Pb[2 * Nc + node]),
+                 pr = cff2_ld(Pb[3 * Nc + node]);
       const float2 wx = lm[s], wy = lm[S + s], wz = lm[2 * S + s], wr = lm[3 * S + s];
-      avr = ff_mad(ffv(wx.x, wx.y), ffv(px.x, px.y), avr);
-      avi = ff_mad(ffv(wx.x, wx.y), ffv(px.z, px.w), avi);
-      avr = ff_mad(ffv(wy.x, wy.y), ffv(py.x, py.y), avr);
-      avi = ff_mad(ffv(wy.x, wy.y), ffv(py.z, py.w), avi);
-      avr = ff_mad(ffv(wz.x, wz.y), ffv(pz.x, pz.y), avr);
-      avi = ff_mad(ffv(wz.x, wz.y), ffv(pz.z, pz.w), avi);
-      arr = ff_mad(ffv(wr.x, wr.y), ffv(pr.x, pr.y), arr);
-      ari = ff_mad(ffv(wr.x, wr.y), ffv(pr.z, pr.w), ari);
+      av = cff2_mad(cff2_both(ffv(wx.x, wx.y)), px, av);
+      av = cff2_mad(cff2_both(ffv(wy.x, wy.y)), py, av);
+      av = cff2_mad(cff2_both(ffv(wz.x, wz.y)), pz, av);
+      ar = cff2_mad(cff2_both(ffv(wr.x, wr.y)), pr, ar);
       if constexpr (MF) {
         const float2 mx = wm[s], my = wm[S + s], mz = wm[2 * S + s];
-        amr = ff_mad(ffv(mx.x, mx.y), ffv(px.x, px.y), amr);
-        ami = ff_mad(ffv(mx.x, mx.y), ffv(px.z, px.w), ami);
-        amr = ff_mad(ffv(my.x, my.y), ffv(py.x, py.y), amr);
-        ami = ff_mad(ffv(my.x, my.y), ffv(py.z, py.w), ami);
-        amr = ff_mad(ffv(mz.x, mz.y), ffv(pz.x, pz.y), amr);
-        ami = ff_mad(ffv(mz.x, mz.y), ffv(pz.z, pz.w), ami);
+        am = cff2_mad(cff2_both(ffv(mx.x, mx.y)), px, am);
+        am = cff2_mad(cff2_both(ffv(my.x, my.y)), py, am);
+        am = cff2_mad(cff2_both(ffv(mz.x, mz.y)), pz, am);
       }
     }
     const float4* xb = x + (long long)b * N;
     for (int e = r0 + lane; e < r1; e += 8) {
-      const float4 v = nval[e], xv = xb[ncol[e]];
-      const ff vr = ffv(v.x, v.y), vi = ffv(v.z, v.w), xr = ffv(xv.x, xv.y), xi = ffv(xv.z, xv.w);
-      anr = ff_mad(vr, xr, anr);
-      anr = ff_mad(ff_neg(vi), xi, anr);
-      ani = ff_mad(vr, xi, ani);
-      ani = ff_mad(vi, xr, ani);
+      const cff2 v = cff2_ld(nval[e]), xv = cff2_ld(xb[ncol[e]]);
+      an = cff2_mad(cff2_re(v), xv, an);
+      an = cff2_mad(cff2_im(v), cff2_times_i(xv), an);
     }
-    // grid part j (fvec av - frho ar): out = an + j t
-    const ff tr = ff_sub(ff_mul(kv, avr), ff_mul(kr, arr));
-    const ff ti = ff_sub(ff_mul(kv, avi), ff_mul(kr, ari));
-    ff outr = ff_sub(anr, ti), outi = ff_add(ani, tr);
-    if constexpr (MF) {
-      outr = ff_sub(outr, ff_mul(km, amr));
-      outi = ff_sub(outi, ff_mul(km, ami));
-    }
+    // an + j (fvec av - frho ar) - fmf am
+    cff2 out = cff2_add(an, cff2_times_i(cff2_dot2(kv, av, kr, ar)));
+    if constexpr (MF) out = cff2_mad(km, am, out);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-      outr = ff_add(outr, ffv(__shfl_xor_sync(0xffffffffu, outr.hi, o, 8), __shfl_xor_sync(0xffffffffu, outr.lo, o, 8)));
-      outi = ff_add(outi, ffv(__shfl_xor_sync(0xffffffffu, outi.hi, o, 8), __shfl_xor_sync(0xffffffffu, outi.lo, o, 8)));
-    }
-    if (live && lane == 0) y[(long long)b * N + m] = make_double2(ff_to_double(outr), ff_to_double(outi));
+    for (int o = 4; o > 0; o >>= 1) out = cff2_add(out, cff2_shfl_xor(out, o, 8));
+    if (live && lane == 0)
+      y[(long long)b * N + m] = make_double2((double)out.hi.x + (double)out.lo.x, (double)out.hi.y + (double)out.lo.y);
   }
 }
 

@@ -219,8 +219,8 @@ int fft_tables(aim_ctx* c) {
       for (int q = 0; q < 2; ++q) {
         const float hi = (float)t64[2 * slot + q];
         t32[2 * slot + q] = hi;
-        tff[4 * slot + 2 * q] = hi;
-        tff[4 * slot + 2 * q + 1] = (float)(t64[2 * slot + q] - (double)hi);
+        tff[4 * slot + q] = hi;
+        tff[4 * slot + 2 + q] = (float)(t64[2 * slot + q] - (double)hi);
       }
     };
     for (int t = 0; t < L; ++t) put(t, t);
