@@ -41,6 +41,7 @@ void free_context(aim_ctx* c) {
   cudaFree(c->pff.pnode_w); cudaFree(c->pff.lam); cudaFree(c->pff.lamM); cudaFree(c->pff.near_val);
   cudaFree(c->pff.xff);
   cudaFree(c->plan_dev);
+  cudaFree(c->rcs_work);
   free_krylov(c);
   profile_free(c);
   cudaFree(c->ngrp_ptr); cudaFree(c->ngrp_col); cudaFree(c->colmask);

@@ -269,6 +269,8 @@ struct aim_ctx {
   aim::PrecData<float> p32;
   aim::FFData pff;
   aim::KrylovWork kw;
+  void* rcs_work = nullptr;   // workspace of aim_rcs kept between calls (rcs.cu)
+  size_t rcs_work_bytes = 0;
   aim::Profiler prof;
   int max_rhs = 1;
   // Multi-instance packs (pack.cu): the pack's internal context has `pack`

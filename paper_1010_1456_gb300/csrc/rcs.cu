@@ -18,6 +18,7 @@
 // take seconds instead of the minutes of FP64 phases.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.h"
@@ -151,7 +152,6 @@ __global__ void k_pack_points(const double* __restrict__ rp, const double2* __re
 // exact for integers |n| < 2^12 (phases below 2.5e4 rad).
 constexpr float kC1 = 6.283203125f, kC2 = -1.7814338207244873e-05f, kC3 = -3.482206523131026e-09f;
 constexpr float kInv2Pi = 0.15915493667125702f;
-constexpr int kFarDirs = 4;      // directions per thread
 constexpr int kFarChunk = 256;   // points staged per shared-memory chunk
 constexpr int kFarRun = 64;      // points summed in FP32 before an FP64 add
 
@@ -171,32 +171,41 @@ __device__ __forceinline__ void far_phase(const ff kr[3], const float* r, float&
   c = __fmaf_rn(-lo, sn, cs);
 }
 
-// N[d][3] += sum over points [p_begin, p_end) of J_p exp(j k rhat_d . r_p),
-// one right-hand side.  Block: 256 threads x kFarDirs directions
-// (d = blockIdx.x * 1024 + i * 256 + threadIdx.x); blockIdx.y picks the
-// point range.  N (FP64 complex [ndir][3]) must be zeroed; partial sums of
-// the point ranges are added atomically.
+// N[b][d][3] += sum over points [p_begin, p_end) of J_p exp(j k rhat_d . r_p)
+// for NR right-hand sides b.  Block: 256 threads x D directions (d =
+// blockIdx.x * 256 D + i * 256 + threadIdx.x); blockIdx.y picks the point
+// range, a multiple of kFarRun.  N (FP64 complex [NR][ndir][3]) must be
+// zeroed; partial sums of the point ranges are added atomically.
+//
+// Bound by FP32 issue: a phase factor takes about 75 instructions, its
+// products with one right-hand side's current 12, so the phase is formed once
+// for all NR (two right-hand sides of a 2 lambda sphere, 87 k points x 8192
+// directions: 5.15 ms one at a time, 2.71 together).  NR D is at most 4, which
+// keeps the FP64 accumulators in registers.
+template <int NR, int D>
 __global__ void __launch_bounds__(256) k_farfield(const float* __restrict__ rff, const float2* __restrict__ J32,
                                                   const double* __restrict__ theta, const double* __restrict__ phi,
                                                   double2* __restrict__ Nacc, long long npts, int ndir,
                                                   long long pts_per_block, double k) {
   __shared__ float sr[kFarChunk][6];
-  __shared__ float2 sj[kFarChunk][3];
-  ff kr[kFarDirs][3];
-  double2 acc[kFarDirs][3];
-  float2 part[kFarDirs][3];
+  __shared__ float2 sj[kFarChunk][NR][3];
+  ff kr[D][3];
+  double2 acc[D][NR][3];
+  float2 part[D][NR][3];
 #pragma unroll
-  for (int i = 0; i < kFarDirs; ++i) {
-    const int d = min(blockIdx.x * (256 * kFarDirs) + i * 256 + threadIdx.x, ndir - 1);
+  for (int i = 0; i < D; ++i) {
+    const int d = min(blockIdx.x * (256 * D) + i * 256 + threadIdx.x, ndir - 1);
     const double st = sin(theta[d]), ct = cos(theta[d]), sp = sin(phi[d]), cp = cos(phi[d]);
     kr[i][0] = ff_from_double(k * st * cp);
     kr[i][1] = ff_from_double(k * st * sp);
     kr[i][2] = ff_from_double(k * ct);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      acc[i][c] = make_double2(0.0, 0.0);
-      part[i][c] = make_float2(0.f, 0.f);
-    }
+    for (int b = 0; b < NR; ++b)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        acc[i][b][c] = make_double2(0.0, 0.0);
+        part[i][b][c] = make_float2(0.f, 0.f);
+      }
   }
   const long long p_begin = blockIdx.y * pts_per_block;
   const long long p_end = min(npts, p_begin + pts_per_block);
@@ -208,51 +217,60 @@ __global__ void __launch_bounds__(256) k_farfield(const float* __restrict__ rff,
 #pragma unroll
       for (int e = 0; e < 6; ++e) sr[threadIdx.x][e] = rff[6 * p + e];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sj[threadIdx.x][c] = J32[3 * p + c];
+      for (int b = 0; b < NR; ++b)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sj[threadIdx.x][b][c] = J32[3 * (b * npts + p) + c];
     }
     __syncthreads();
     for (int q = 0; q < cnt; ++q) {
-      const float2 jx = sj[q][0], jy = sj[q][1], jz = sj[q][2];
 #pragma unroll
-      for (int i = 0; i < kFarDirs; ++i) {
+      for (int i = 0; i < D; ++i) {
         float c, s;
         far_phase(kr[i], sr[q], c, s);
-        part[i][0].x = __fmaf_rn(jx.x, c, __fmaf_rn(-jx.y, s, part[i][0].x));
-        part[i][0].y = __fmaf_rn(jx.x, s, __fmaf_rn(jx.y, c, part[i][0].y));
-        part[i][1].x = __fmaf_rn(jy.x, c, __fmaf_rn(-jy.y, s, part[i][1].x));
-        part[i][1].y = __fmaf_rn(jy.x, s, __fmaf_rn(jy.y, c, part[i][1].y));
-        part[i][2].x = __fmaf_rn(jz.x, c, __fmaf_rn(-jz.y, s, part[i][2].x));
-        part[i][2].y = __fmaf_rn(jz.x, s, __fmaf_rn(jz.y, c, part[i][2].y));
+#pragma unroll
+        for (int b = 0; b < NR; ++b)
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            const float2 j = sj[q][b][e];
+            part[i][b][e].x = __fmaf_rn(j.x, c, __fmaf_rn(-j.y, s, part[i][b][e].x));
+            part[i][b][e].y = __fmaf_rn(j.x, s, __fmaf_rn(j.y, c, part[i][b][e].y));
+          }
       }
       if ((q & (kFarRun - 1)) == kFarRun - 1 || q == cnt - 1) {
 #pragma unroll
-        for (int i = 0; i < kFarDirs; ++i)
+        for (int i = 0; i < D; ++i)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            acc[i][c].x += (double)part[i][c].x;
-            acc[i][c].y += (double)part[i][c].y;
-            part[i][c] = make_float2(0.f, 0.f);
-          }
+          for (int b = 0; b < NR; ++b)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              acc[i][b][c].x += (double)part[i][b][c].x;
+              acc[i][b][c].y += (double)part[i][b][c].y;
+              part[i][b][c] = make_float2(0.f, 0.f);
+            }
       }
     }
   }
 #pragma unroll
-  for (int i = 0; i < kFarDirs; ++i) {
-    const int d = blockIdx.x * (256 * kFarDirs) + i * 256 + threadIdx.x;
+  for (int i = 0; i < D; ++i) {
+    const int d = blockIdx.x * (256 * D) + i * 256 + threadIdx.x;
     if (d >= ndir) continue;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      atomicAdd(&Nacc[3 * (long long)d + c].x, acc[i][c].x);
-      atomicAdd(&Nacc[3 * (long long)d + c].y, acc[i][c].y);
-    }
+    for (int b = 0; b < NR; ++b)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        atomicAdd(&Nacc[3 * ((long long)b * ndir + d) + c].x, acc[i][b][c].x);
+        atomicAdd(&Nacc[3 * ((long long)b * ndir + d) + c].y, acc[i][b][c].y);
+      }
   }
 }
 
-// (N_theta, N_phi) [ndir] from the Cartesian far field N [ndir][3]
+// (N_theta, N_phi) [ndir] from the Cartesian far field N [ndir][3]; blockIdx.y: right-hand side
 __global__ void k_far_project(const double2* __restrict__ Nacc, const double* __restrict__ theta,
                               const double* __restrict__ phi, double2* __restrict__ out, int ndir) {
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= ndir) return;
+  Nacc += 3LL * blockIdx.y * ndir;
+  out += 2LL * blockIdx.y * ndir;
   const double st = sin(theta[d]), ct = cos(theta[d]), sp = sin(phi[d]), cp = cos(phi[d]);
   const double2 nx = Nacc[3 * (long long)d], ny = Nacc[3 * (long long)d + 1], nz = Nacc[3 * (long long)d + 2];
   out[2 * (long long)d] = make_double2(ct * cp * nx.x + ct * sp * ny.x - st * nz.x, ct * cp * nx.y + ct * sp * ny.y - st * nz.y);
@@ -275,26 +293,76 @@ int rhs_planewave(aim_ctx* c, int nrhs, const double* khat, const double* pol, d
   return AIM_OK;
 }
 
+// Far fields of NR right-hand sides in one launch.  Point ranges of at least one FP32 run are
+// split until every SM has about four blocks, each thread first giving up its extra directions
+// (a plate of 1.5 k points and 1152 directions took 1.2 ms a right-hand side on two blocks).
+template <int NR>
+static int far_fields(aim_ctx* c, const float* rff, const float2* J32, const double* dang, double2* Nacc,
+                      long long npts, int ndir) {
+  constexpr int DMAX = 4 / NR;
+  const long long runs = (npts + kFarRun - 1) / kFarRun;
+  const auto launch = [&](auto dirs) -> int {
+    constexpr int D = decltype(dirs)::value;
+    const int bx = (ndir + 256 * D - 1) / (256 * D);
+    const long long by = std::min(runs, std::max<long long>(1, (4LL * 152 + bx - 1) / bx));
+    const long long ppb = (runs + by - 1) / by * kFarRun;
+    AIM_LAUNCH(c, "k_farfield", (k_farfield<NR, D><<<dim3(bx, (unsigned)((npts + ppb - 1) / ppb)), 256, 0, c->stream>>>(
+                                    rff, J32, dang, dang + ndir, Nacc, npts, ndir, ppb, c->k)));
+    return launch_check(c, "k_farfield");
+  };
+  const bool wide = (ndir + 256 * DMAX - 1) / (256 * DMAX) * (runs / 4) >= 4 * 152;
+  if constexpr (DMAX > 1)
+    if (wide) return launch(std::integral_constant<int, DMAX>{});
+  return launch(std::integral_constant<int, 1>{});
+}
+
+// Workspace kept with the context between calls up to this size (a call synchronises, so it is
+// idle in between); larger ones, and those of a context with a memory budget, live for the call.
+constexpr size_t kRcsKeep = 64ull << 20;
+
 int rcs(aim_ctx* c, const double2* X, int nrhs, int ndir, const double* theta, const double* phi, double* sig_tt,
         double* sig_pp) {
   AIM_TRY(upload_rules());
   const int nq = kFarRule * kFarRule;
   const long long npts = (long long)c->nt * nq;
-  double2* J = nullptr;
-  double *rp = nullptr, *dang = nullptr;
-  double2 *Nacc = nullptr, *out = nullptr;
-  float* rff = nullptr;
-  float2* J32 = nullptr;
-  AIM_CUDA_TRY(cudaMallocAsync(&J, sizeof(double2) * 3 * npts * nrhs, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&rp, sizeof(double) * 3 * npts, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&rff, sizeof(float) * 6 * npts, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&J32, sizeof(float2) * 3 * npts * nrhs, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&dang, sizeof(double) * 2 * ndir, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&Nacc, sizeof(double2) * 3 * (size_t)ndir * nrhs, c->stream));
-  AIM_CUDA_TRY(cudaMallocAsync(&out, sizeof(double2) * 2 * (size_t)ndir * nrhs, c->stream));
-  AIM_CUDA_TRY(cudaMemsetAsync(J, 0, sizeof(double2) * 3 * npts * nrhs, c->stream));
-  AIM_CUDA_TRY(cudaMemsetAsync(rp, 0, sizeof(double) * 3 * npts, c->stream));
-  AIM_CUDA_TRY(cudaMemsetAsync(Nacc, 0, sizeof(double2) * 3 * (size_t)ndir * nrhs, c->stream));
+  // one block of memory: what must start as zero first
+  size_t total = 0;
+  const auto take = [&](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t oJ = take(sizeof(double2) * 3 * npts * nrhs), oN = take(sizeof(double2) * 3 * (size_t)ndir * nrhs),
+               orp = take(sizeof(double) * 3 * npts), zeroed = total, orff = take(sizeof(float) * 6 * npts),
+               oJ32 = take(sizeof(float2) * 3 * npts * nrhs), oang = take(sizeof(double) * 2 * ndir),
+               oout = take(sizeof(double2) * 2 * (size_t)ndir * nrhs);
+  struct Temp {  // freed on every way out
+    void* p = nullptr;
+    cudaStream_t st;
+    ~Temp() {
+      if (p) cudaFreeAsync(p, st);
+    }
+  } tmp;
+  tmp.st = c->stream;
+  char* base = nullptr;
+  if (total <= kRcsKeep && c->opts.mem_budget == 0) {
+    if (c->rcs_work_bytes < total) {
+      cudaFree(c->rcs_work);
+      c->rcs_work = nullptr;
+      c->rcs_work_bytes = 0;
+      AIM_CUDA_TRY(cudaMalloc(&c->rcs_work, total));
+      c->rcs_work_bytes = total;
+    }
+    base = (char*)c->rcs_work;
+  } else {
+    AIM_CUDA_TRY(cudaMallocAsync(&tmp.p, total, c->stream));
+    base = (char*)tmp.p;
+  }
+  double2 *J = (double2*)(base + oJ), *Nacc = (double2*)(base + oN), *out = (double2*)(base + oout);
+  double *rp = (double*)(base + orp), *dang = (double*)(base + oang);
+  float* rff = (float*)(base + orff);
+  float2* J32 = (float2*)(base + oJ32);
+  AIM_CUDA_TRY(cudaMemsetAsync(base, 0, zeroed, c->stream));
   AIM_CUDA_TRY(cudaMemcpyAsync(dang, theta, sizeof(double) * ndir, cudaMemcpyHostToDevice, c->stream));
   AIM_CUDA_TRY(cudaMemcpyAsync(dang + ndir, phi, sizeof(double) * ndir, cudaMemcpyHostToDevice, c->stream));
   const long long nthr = (long long)c->N * 2 * nq;
@@ -304,32 +372,27 @@ int rcs(aim_ctx* c, const double2* X, int nrhs, int ndir, const double* theta, c
   AIM_LAUNCH(c, "k_pack_points", k_pack_points<<<(unsigned)std::min<long long>((npts + 255) / 256, 152LL * 16), 256, 0,
                                                   c->stream>>>(rp, J, rff, J32, npts, nrhs));
   AIM_TRY(launch_check(c, "k_pack_points"));
-  // direction tiles x point ranges: at least about four blocks per SM in total
-  const int per_block = 256 * kFarDirs;
-  const int bx = (ndir + per_block - 1) / per_block;
-  long long by = std::max<long long>(1, (4LL * 152 + bx - 1) / bx);
-  by = std::min<long long>(by, std::max<long long>(1, npts / (4 * kFarChunk)));
-  long long ppb = (npts + by - 1) / by;
-  ppb = (ppb + kFarChunk - 1) / kFarChunk * kFarChunk;
-  by = (npts + ppb - 1) / ppb;
-  for (int b = 0; b < nrhs; ++b) {
-    AIM_LAUNCH(c, "k_farfield", (k_farfield<<<dim3(bx, (unsigned)by), 256, 0, c->stream>>>(
-                                    rff, J32 + (size_t)b * npts * 3, dang, dang + ndir, Nacc + (size_t)b * ndir * 3,
-                                    npts, ndir, ppb, c->k)));
-    AIM_TRY(launch_check(c, "k_farfield"));
-    AIM_LAUNCH(c, "k_far_project", (k_far_project<<<(ndir + 255) / 256, 256, 0, c->stream>>>(
+  for (int b = 0; b < nrhs;) {
+    const float2* Jb = J32 + (size_t)b * npts * 3;
+    double2* Nb = Nacc + (size_t)b * ndir * 3;
+    if (nrhs - b >= 4) {
+      AIM_TRY(far_fields<4>(c, rff, Jb, dang, Nb, npts, ndir));
+      b += 4;
+    } else if (nrhs - b >= 2) {
+      AIM_TRY(far_fields<2>(c, rff, Jb, dang, Nb, npts, ndir));
+      b += 2;
+    } else {
+      AIM_TRY(far_fields<1>(c, rff, Jb, dang, Nb, npts, ndir));
+      b += 1;
+    }
+  }
+  for (int b = 0; b < nrhs; b += 32768) {
+    AIM_LAUNCH(c, "k_far_project", (k_far_project<<<dim3((ndir + 255) / 256, std::min(32768, nrhs - b)), 256, 0, c->stream>>>(
                                        Nacc + (size_t)b * ndir * 3, dang, dang + ndir, out + (size_t)b * ndir * 2, ndir)));
     AIM_TRY(launch_check(c, "k_far_project"));
   }
   std::vector<double2> h((size_t)2 * ndir * nrhs);
   AIM_CUDA_TRY(cudaMemcpyAsync(h.data(), out, sizeof(double2) * h.size(), cudaMemcpyDeviceToHost, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(J, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(rp, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(rff, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(J32, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(dang, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(Nacc, c->stream));
-  AIM_CUDA_TRY(cudaFreeAsync(out, c->stream));
   AIM_CUDA_TRY(cudaStreamSynchronize(c->stream));
   const double fac = c->k * c->k * kEta0 * kEta0 / (4.0 * kPi);
   for (int b = 0; b < nrhs; ++b)
