@@ -173,15 +173,19 @@ struct KrylovWork {
   double2* r = nullptr;      // [B][N]
   double2* H = nullptr;      // [m][B][m+1] Hessenberg columns (column j of every RHS is contiguous)
   double2* partial = nullptr;// [B][nblk][m+1+kDotGroup] partial dots
+  double2* hcur = nullptr;   // [B][m+1+kDotGroup] the dots of the current Gram-Schmidt pass
+  unsigned* cnt = nullptr;   // [B][vector groups] finished blocks of the dot kernel (zero between launches)
   double2* y = nullptr;      // [B][m] least-squares solution of the cycle
   double* nrm = nullptr;     // [B] norms, [B] spare, then [B][nblk] norm partials
   double* bnorm = nullptr;   // [B]
   double2* h_H = nullptr;    // pinned host copy of H columns
   int* active = nullptr;     // [B]
   int* reorth = nullptr;     // [B] second Gram-Schmidt pass needed for the current column
-  int* jdev = nullptr;       // current Arnoldi column (read by the step's kernels)
+  int* jdev = nullptr;       // current Arnoldi column (read by the step's kernels), then the blocks of the
+                             // normalising kernel that have finished (zero between launches)
   int m = 0;
   int nblk = 0;              // blocks per right-hand side of the norm kernel
+  int nblk_upd = 0;          // blocks per right-hand side of the update kernel
   int nblk_dot = 0;          // blocks per right-hand side and vector group of the dot kernel
   // CUDA graph of one Arnoldi step (per precision and batch size), captured
   // on a private stream (the legacy default stream cannot be captured)

@@ -22,6 +22,7 @@
 namespace aim {
 
 constexpr int kDotGroup = 8;  // basis vectors per pass of the dot kernel
+constexpr int kUpdThreads = 128;   // threads per block of the update kernel
 constexpr int kTfqmrVecs = 9;      // vectors per right-hand side of the TFQMR iteration
 constexpr int kTfqmrScalars = 8;   // complex scalars per right-hand side of the TFQMR iteration
 
@@ -32,41 +33,59 @@ __device__ __forceinline__ double2 cfma_conj(double2 a, double2 b, double2 acc) 
   return acc;
 }
 
-template <int NV>
-__device__ __forceinline__ void block_reduce_store(double2* v, double2* out, int stride) {
+// Sums of kDotGroup complex values over the block; threads i < kDotGroup store value i at out[i].
+// A warp halves its values at every step (a lane keeps the half its bit names and receives the
+// partner's share of it): 16 FP64 additions a thread where reducing each of the 16 reals by itself
+// took 80, on a pipe that retires two a clock per SM.
+__device__ __forceinline__ void block_reduce_store(double2* v, double2* out) {
+  static_assert(kDotGroup == 8, "three halving steps");
   __shared__ double2 red[32][kDotGroup];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-  for (int i = 0; i < NV; ++i)
-    for (int o = 16; o > 0; o >>= 1) {
-      v[i].x += __shfl_xor_sync(0xffffffffu, v[i].x, o);
-      v[i].y += __shfl_xor_sync(0xffffffffu, v[i].y, o);
+  for (int h = kDotGroup / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < kDotGroup / 2; ++i) {
+      if (i >= h) break;
+      const double2 keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+      v[i].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, o);
+      v[i].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, o);
     }
-  if (lane == 0)
-    for (int i = 0; i < NV; ++i) red[warp][i] = v[i];
+  }
+  // lane bits 4, 3, 2 name the value; bits 1, 0 hold shares of it
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) {
+    v[0].x += __shfl_xor_sync(0xffffffffu, v[0].x, o);
+    v[0].y += __shfl_xor_sync(0xffffffffu, v[0].y, o);
+  }
+  if ((lane & 3) == 0) red[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = v[0];
   __syncthreads();
-  if (threadIdx.x < NV) {
+  if (threadIdx.x < kDotGroup) {
     double2 s = make_double2(0, 0);
     for (int w = 0; w < nw; ++w) {
       s.x += red[w][threadIdx.x].x;
       s.y += red[w][threadIdx.x].y;
     }
-    out[threadIdx.x * stride] = s;
+    out[threadIdx.x] = s;
   }
-  __syncthreads();
 }
 
 // Every kernel of the Arnoldi step reads the column index j from device
 // memory (jdev), so one captured CUDA graph serves every step of a cycle.
 
-// Pass `pass` of classical Gram-Schmidt for column j, partial dot products:
-// partial[b][blk][i] = sum over block blk's chunk of conj(V[b][i]) . w[b],
-// i <= j; on the first pass the slot i = j + 1 receives |w|^2 (the norm before
-// orthogonalising, for the re-orthogonalisation test).  Grid: (vector groups
-// of kDotGroup, nblk, B); blocks past the column's vectors, and the second
-// pass of right-hand sides that need no re-orthogonalisation, return at once.
+// Pass `pass` of classical Gram-Schmidt for column j: h[b][i] = sum of
+// conj(V[b][i]) . w[b], i <= j; on the first pass the slot i = j + 1 receives
+// |w|^2 (the norm before orthogonalising, for the re-orthogonalisation test).
+// Grid: (vector groups of kDotGroup, nblk, B); blocks past the column's
+// vectors, and the second pass of right-hand sides that need no
+// re-orthogonalisation, return at once.  A block sums its chunk of N; the last
+// block of a (group, right-hand side) to finish adds the chunks' sums in
+// their order, so the result does not depend on which block that is (cnt
+// counts them and is left at zero).  Bound by the FP64 pipe (4 FMAs per
+// element and vector, two a clock per SM).
 __global__ void __launch_bounds__(256) k_dots(const double2* __restrict__ V, const double2* __restrict__ w,
-                                              double2* __restrict__ partial, const int* __restrict__ jdev,
+                                              double2* __restrict__ partial, double2* __restrict__ h,
+                                              unsigned* __restrict__ cnt, const int* __restrict__ jdev,
                                               const int* __restrict__ reorth, int N, int ldv_vec, int nblk, int ldp,
                                               int pass) {
   const int b = blockIdx.z, blk = blockIdx.y, i0 = blockIdx.x * kDotGroup;
@@ -87,35 +106,54 @@ __global__ void __launch_bounds__(256) k_dots(const double2* __restrict__ V, con
     for (int i = 0; i < kDotGroup; ++i)
       if (i < ni) acc[i] = cfma_conj(i0 + i < nvec ? Vb[(long long)(i0 + i) * N + n] : wv, wv, acc[i]);
   }
-  block_reduce_store<kDotGroup>(acc, partial + ((long long)b * nblk + blk) * ldp + i0, 1);
+  const double2* pb = partial + (long long)b * nblk * ldp + i0;
+  block_reduce_store(acc, partial + ((long long)b * nblk + blk) * ldp + i0);
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned* c = cnt + (long long)b * gridDim.x + blockIdx.x;
+    last = atomicAdd(c, 1u) == (unsigned)nblk - 1;
+    if (last) *c = 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // warp i: slot i0 + i; lanes take every 32nd chunk, then combine
+  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (i >= ni) return;
+  double2 t = make_double2(0, 0);
+  for (int q = lane; q < nblk; q += 32) {
+    const double2 p = __ldcg(pb + (long long)q * ldp + i);
+    t.x += p.x;
+    t.y += p.y;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+  }
+  if (lane == 0) h[(long long)b * ldp + i0 + i] = t;
 }
 
-// w[b] -= sum_{i <= j} h[b][i] V[b][i], where every block first sums the dot
-// kernel's partials itself (h[i] = sum over blk of partial[b][blk][i], in a
-// fixed order, so every block holds the same values) and block 0 stores the
-// Hessenberg column: H[j][b][i] = h (first pass) or += h (second pass).  On
-// the first pass slot i = j + 1 holds |w|^2 before orthogonalising, and
-// block 0 evaluates the re-orthogonalisation test of Daniel, Gragg, Kaufman
-// and Stewart, |w1|^2 = |w0|^2 - |h|^2 < |w0|^2 / 2; the second pass runs
-// only where it holds.
-__global__ void __launch_bounds__(256) k_update(const double2* __restrict__ V, double2* __restrict__ w,
-                                                const double2* __restrict__ partial, double2* __restrict__ H,
-                                                int* __restrict__ reorth, const int* __restrict__ jdev, int N,
-                                                int ldv_vec, int m, int B, int nblk, int ldp, int pass) {
+// w[b] -= sum_{i <= j} h[b][i] V[b][i], with the sums of k_dots; block 0
+// stores the Hessenberg column: H[j][b][i] = h (first pass) or += h (second
+// pass).  On the first pass slot i = j + 1 holds |w|^2 before orthogonalising,
+// and block 0 evaluates the re-orthogonalisation test of Daniel, Gragg,
+// Kaufman and Stewart, |w1|^2 = |w0|^2 - |h|^2 < |w0|^2 / 2; the second pass
+// runs only where it holds.  Every block leaves its part of |w|^2 in
+// npart[b][block] (a second pass that does not run leaves the first's).
+__global__ void __launch_bounds__(kUpdThreads) k_update(const double2* __restrict__ V, double2* __restrict__ w,
+                                                        const double2* __restrict__ hcur, double2* __restrict__ H,
+                                                        double* __restrict__ npart, int* __restrict__ reorth,
+                                                        const int* __restrict__ jdev, int N, int ldv_vec, int m,
+                                                        int B, int ldp, int pass) {
   __shared__ double2 hs[256];
   const int b = blockIdx.y;
   if (pass == 1 && !reorth[b]) return;
   const int j = *jdev, nvec = j + 1;
   const int nslot = pass == 0 ? nvec + 1 : nvec;
-  for (int i = threadIdx.x; i < nslot; i += blockDim.x) {
-    double2 t = make_double2(0, 0);
-    for (int blk = 0; blk < nblk; ++blk) {
-      const double2 p = partial[((long long)b * nblk + blk) * ldp + i];
-      t.x += p.x;
-      t.y += p.y;
-    }
-    hs[i] = t;
-  }
+  for (int i = threadIdx.x; i < nslot; i += blockDim.x) hs[i] = hcur[(long long)b * ldp + i];
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
@@ -136,14 +174,27 @@ __global__ void __launch_bounds__(256) k_update(const double2* __restrict__ V, d
   }
   const double2* Vb = V + (long long)b * ldv_vec * N;
   double2* wb = w + (long long)b * N;
+  double s2 = 0.0;
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
     double2 acc = wb[n];
+#pragma unroll 8
     for (int i = 0; i < nvec; ++i) {
       const double2 v = Vb[(long long)i * N + n], h = hs[i];
       acc.x -= h.x * v.x - h.y * v.y;
       acc.y -= h.x * v.y + h.y * v.x;
     }
     wb[n] = acc;
+    s2 += acc.x * acc.x + acc.y * acc.y;
+  }
+  __shared__ double red[kUpdThreads / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < kUpdThreads / 32; ++q) t += red[q];
+    npart[(long long)b * gridDim.x + blockIdx.x] = t;
   }
 }
 
@@ -190,13 +241,17 @@ __global__ void k_scale(const double2* __restrict__ src, double2* __restrict__ d
   }
 }
 
-// End of the step: |w| from the norm kernel's partial sums (every block
-// reduces them in the same order), V[b][j + 1] = w[b] / |w|; block 0 stores
-// |w| as the subdiagonal H[j][b][j + 1].
+// End of the step: |w| from the update kernel's partial sums (every block
+// reduces them in the same order), V[b][j + 1] = w[b] / |w| and the next
+// product's input z = dinv .* V[b][j + 1] (precision R); block 0 stores |w| as
+// the subdiagonal H[j][b][j + 1].  The last block to finish moves the column
+// index on (jdev[1] counts the blocks and is left at zero): all have read it.
+template <typename R>
 __global__ void __launch_bounds__(256) k_normalize(const double2* __restrict__ w, double2* __restrict__ V,
                                                    const double* __restrict__ npart, double2* __restrict__ H,
-                                                   const int* __restrict__ jdev, int N, long long ldv, int nblk,
-                                                   int m, int B) {
+                                                   int* __restrict__ jdev, int N, long long ldv, int nblk, int m,
+                                                   int B, const double2* __restrict__ dinv, long long ldd,
+                                                   cplx<R>* __restrict__ z) {
   __shared__ double red[8];
   __shared__ double nrm_s;
   const int b = blockIdx.y;
@@ -211,19 +266,25 @@ __global__ void __launch_bounds__(256) k_normalize(const double2* __restrict__ w
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) u += red[i];
     nrm_s = sqrt(u);
     if (blockIdx.x == 0) H[((long long)j * B + b) * (m + 1) + j + 1] = make_double2(nrm_s, 0.0);
+    if (atomicAdd(jdev + 1, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+      jdev[1] = 0;
+      jdev[0] = j + 1;
+    }
   }
   __syncthreads();
   const double s = nrm_s > 0.0 ? 1.0 / nrm_s : 0.0;
   double2* dst = V + (long long)b * ldv + (long long)(j + 1) * N;
+  const double2* db = dinv + (long long)b * ldd;
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
     double2 v = w[(long long)b * N + n];
     v.x *= s;
     v.y *= s;
     dst[n] = v;
+    const double2 d = db[n];
+    z[(long long)b * N + n] = cmake<cplx<R>>(v.x * d.x - v.y * d.y, v.x * d.y + v.y * d.x);
   }
 }
 
-__global__ void k_next_j(int* jdev) { *jdev += 1; }
 __global__ void k_set_j(int* jdev, int j) { *jdev = j; }
 
 // z = dinv .* V_j, in precision R (dinv: row b at b * ldd; ldd = 0 shares one diagonal)
@@ -292,9 +353,12 @@ int alloc_krylov(aim_ctx* c) {
   k.m = m;
   // norm kernel: about four blocks per SM over all right-hand sides, at least 256 elements per block
   k.nblk = std::max(1, std::min((4 * 152 + B - 1) / B, (N + 255) / 256));
-  // dot kernel: at least 1024 elements per block, about two blocks per SM per vector group
-  k.nblk_dot = std::max(1, std::min((2 * 152 + B - 1) / B, (N + 1023) / 1024));
-  const int nb = std::max(k.nblk, k.nblk_dot);
+  // dot kernel: at least 512 elements per block, about two blocks per SM per vector group (its
+  // FP64 work has to reach every SM: with 1024 the second vector group of two right-hand sides of
+  // 14,520 unknowns was the first to fill the GPU)
+  k.nblk_dot = std::max(1, std::min((2 * 152 + B - 1) / B, (N + 511) / 512));
+  k.nblk_upd = std::min(1024, (N + kUpdThreads - 1) / kUpdThreads);
+  const int nb = std::max(std::max(k.nblk, k.nblk_dot), k.nblk_upd);
   const size_t vec = (size_t)N * sizeof(double2);
   AIM_CUDA_TRY(cudaMalloc(&k.V, vec * B * slots));
   k.slots = slots;
@@ -307,7 +371,12 @@ int alloc_krylov(aim_ctx* c) {
   AIM_CUDA_TRY(cudaMalloc(&k.bnorm, sizeof(double) * B));
   AIM_CUDA_TRY(cudaMalloc(&k.active, sizeof(int) * B));
   AIM_CUDA_TRY(cudaMalloc(&k.reorth, sizeof(int) * B));
-  AIM_CUDA_TRY(cudaMalloc(&k.jdev, sizeof(int)));
+  AIM_CUDA_TRY(cudaMalloc(&k.hcur, sizeof(double2) * B * (m + 1 + kDotGroup)));
+  const size_t ncnt = sizeof(unsigned) * B * ((m + 2 + kDotGroup - 1) / kDotGroup);
+  AIM_CUDA_TRY(cudaMalloc(&k.cnt, ncnt));
+  AIM_CUDA_TRY(cudaMemsetAsync(k.cnt, 0, ncnt, c->stream));
+  AIM_CUDA_TRY(cudaMalloc(&k.jdev, 2 * sizeof(int)));
+  AIM_CUDA_TRY(cudaMemsetAsync(k.jdev, 0, 2 * sizeof(int), c->stream));
   AIM_CUDA_TRY(cudaMallocHost(&k.h_H, sizeof(double2) * (size_t)B * (m + 1) * m));
   AIM_CUDA_TRY(cudaStreamCreateWithFlags(&k.cap_stream, cudaStreamNonBlocking));
   return AIM_OK;
@@ -324,7 +393,7 @@ void free_krylov(aim_ctx* c) {
   if (k.cap_stream) cudaStreamDestroy(k.cap_stream);
   cudaFree(k.V); cudaFree(k.w); cudaFree(k.r); cudaFree(k.H); cudaFree(k.partial);
   cudaFree(k.y); cudaFree(k.nrm); cudaFree(k.bnorm);
-  cudaFree(k.active); cudaFree(k.reorth); cudaFree(k.jdev);
+  cudaFree(k.active); cudaFree(k.reorth); cudaFree(k.jdev); cudaFree(k.hcur); cudaFree(k.cnt);
   if (k.h_H) cudaFreeHost(k.h_H);
   k = KrylovWork{};
 }
@@ -353,38 +422,48 @@ struct Solver {
     return chk("k_sqrt_sum");
   }
 
-  // One Arnoldi step for the column j held in device memory (k.jdev):
-  // w = Z~ (dinv .* v_j) in `precision`, CGS with selective second pass into
-  // the Hessenberg column H[j], v_{j+1} = w / |w|, j += 1.
-  int step(int precision) {
-    if (precision == AIM_C64) {
+  // The product's input of the column held in k.jdev: dinv .* v_j.  Called once per cycle; every
+  // step leaves the next one's.
+  int precond(int precision) {
+    if (precision == AIM_C64)
       AIM_LAUNCH(c, "k_precond", k_precond<float><<<vgrid(), 256, 0, st>>>(k.V, c->dinv64, c->p32.xbuf, k.jdev, N, ldV(),
                                                                            c->dinv_ld));
-      AIM_TRY(chk("k_precond"));
+    else
+      AIM_LAUNCH(c, "k_precond", k_precond<double><<<vgrid(), 256, 0, st>>>(k.V, c->dinv64, c->p64.xbuf, k.jdev, N, ldV(),
+                                                                            c->dinv_ld));
+    return chk("k_precond");
+  }
+
+  // One Arnoldi step for the column j held in device memory (k.jdev):
+  // w = Z~ (dinv .* v_j) in `precision`, CGS with selective second pass into
+  // the Hessenberg column H[j], v_{j+1} = w / |w|, dinv .* v_{j+1}, j += 1.
+  int step(int precision) {
+    if (precision == AIM_C64) {
       AIM_TRY(matvec(c, c->p32.xbuf, c->p32.ybuf, B, AIM_C64));
       AIM_TRY(convert_c64_to_c128(c, c->p32.ybuf, k.w, (int64_t)B * N));
     } else {
-      AIM_LAUNCH(c, "k_precond", k_precond<double><<<vgrid(), 256, 0, st>>>(k.V, c->dinv64, c->p64.xbuf, k.jdev, N, ldV(),
-                                                                            c->dinv_ld));
-      AIM_TRY(chk("k_precond"));
       AIM_TRY(matvec(c, c->p64.xbuf, k.w, B, precision));
     }
     const int ldp = m + 1 + kDotGroup;
     const dim3 dgrid((m + 2 + kDotGroup - 1) / kDotGroup, k.nblk_dot, B);
+    const dim3 ugrid((unsigned)k.nblk_upd, B);
     for (int pass = 0; pass < 2; ++pass) {
-      AIM_LAUNCH(c, "k_dots", k_dots<<<dgrid, 256, 0, st>>>(k.V, k.w, k.partial, k.jdev, k.reorth, N, m + 1,
-                                                            k.nblk_dot, ldp, pass));
+      AIM_LAUNCH(c, "k_dots", k_dots<<<dgrid, 256, 0, st>>>(k.V, k.w, k.partial, k.hcur, k.cnt, k.jdev, k.reorth, N,
+                                                            m + 1, k.nblk_dot, ldp, pass));
       AIM_TRY(chk("k_dots"));
-      AIM_LAUNCH(c, "k_update", k_update<<<vgrid(), 256, 0, st>>>(k.V, k.w, k.partial, k.H, k.reorth, k.jdev, N,
-                                                                  m + 1, m, B, k.nblk_dot, ldp, pass));
+      AIM_LAUNCH(c, "k_update", k_update<<<ugrid, kUpdThreads, 0, st>>>(k.V, k.w, k.hcur, k.H, npart, k.reorth, k.jdev,
+                                                                        N, m + 1, m, B, ldp, pass));
       AIM_TRY(chk("k_update"));
     }
-    AIM_TRY(norm_partials(k.w, N));
-    AIM_LAUNCH(c, "k_normalize", k_normalize<<<vgrid(), 256, 0, st>>>(k.w, k.V, npart, k.H, k.jdev, N, ldV(), k.nblk,
-                                                                     m, B));
-    AIM_TRY(chk("k_normalize"));
-    AIM_LAUNCH(c, "k_next_j", k_next_j<<<1, 1, 0, st>>>(k.jdev));
-    return chk("k_next_j");
+    if (precision == AIM_C64)
+      AIM_LAUNCH(c, "k_normalize", k_normalize<float><<<vgrid(), 256, 0, st>>>(
+                                       k.w, k.V, npart, k.H, k.jdev, N, ldV(), k.nblk_upd, m, B, c->dinv64,
+                                       c->dinv_ld, c->p32.xbuf));
+    else
+      AIM_LAUNCH(c, "k_normalize", k_normalize<double><<<vgrid(), 256, 0, st>>>(
+                                       k.w, k.V, npart, k.H, k.jdev, N, ldV(), k.nblk_upd, m, B, c->dinv64,
+                                       c->dinv_ld, c->p64.xbuf));
+    return chk("k_normalize");
   }
 
   // The step as a CUDA graph (captured on first use for this precision and
@@ -546,6 +625,7 @@ static int solve_gmres(aim_ctx* c, const double2* V, double2* X, int nrhs, doubl
     AIM_TRY(s.chk("k_scale"));
     AIM_LAUNCH(c, "k_set_j", k_set_j<<<1, 1, 0, c->stream>>>(k.jdev, 0));
     AIM_TRY(s.chk("k_set_j"));
+    AIM_TRY(s.precond(prec));
     for (int b = 0; b < nrhs; ++b) lsq[b].start(beta[b]);
     int kk = 0, done_cols = 0;
     // Hessenberg columns done_cols .. kk-1 to the host, Givens rotations; true when every active RHS is converged
