@@ -9,8 +9,8 @@
 //
 // The projection is a gather over each grid node's list of (basis, weight)
 // entries, built at setup, so it needs no atomics and is deterministic.  The
-// interpolation and the near row of a basis function are handled by one
-// 8-lane group: the lanes split the stencil nodes and the near entries and
+// interpolation and the near row of a basis function are handled by one group
+// of 8 or 32 lanes: the lanes split the stencil nodes and the near entries and
 // reduce with warp shuffles.
 //
 // Modes: M32 (complex64, FP32 accumulation) and M64 (complex128 throughout);
@@ -93,8 +93,11 @@ struct ProjTasks {
 // start).  The next task's list bounds are loaded while the current one is
 // summed, and the right-hand sides go in chunks of BC: an entry's weights
 // and column are loaded once per chunk and its BC gathers of x are
-// independent loads.
-template <class MD, int BC>
+// independent loads.  U entries are in flight per lane: two where the tasks
+// are a single wave of blocks, which then only wait for their loads (a 5
+// lambda plate, 4 right-hand sides: 10.9 -> 9.0 us), one beyond, where the
+// registers of a second cost resident warps (7 lambda sphere: 107 us, 127).
+template <class MD, int BC, int U>
 __global__ void __launch_bounds__(256) proj_gather(const cplx<typename MD::R>* __restrict__ x, typename MD::S* __restrict__ Q,
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ mm,
                                                    const typename MD::R* __restrict__ w, int N, long long Nc, int nrhs,
@@ -129,6 +132,7 @@ __global__ void __launch_bounds__(256) proj_gather(const cplx<typename MD::R>* _
       for (int q = 0; q < BC; ++q)
 #pragma unroll
         for (int c = 0; c < 4; ++c) a[q][c] = cmake<C>(0, 0);
+#pragma unroll(U)
       for (int e = e0 + lane; e < e1; e += 4) {
         const W4<R> ww = load_w4(w, e);
         const C* xc = x + mm[e];
@@ -173,9 +177,14 @@ __device__ __forceinline__ void stencil_offsets_smem(int* s_off, int S, int P, i
 }
 constexpr int kMaxStencil = 216;
 
-// 8 lanes per basis function.
-template <class MD, bool MF>
-__global__ void __launch_bounds__(256) interp_near(const typename MD::S* __restrict__ Phi,
+// W lanes per basis function, BC right-hand sides at a time.  Bound by the
+// latency of its gathers (stencil nodes of Phi, columns of x), so a chunk of
+// right-hand sides keeps BC times as many in flight and reads the weights, the
+// near entries and their columns once for all of them (16 lambda sphere, 8
+// right-hand sides: 1.82 -> 1.38 ms); a small body takes a whole warp per basis function, which leaves one or two rounds of gathers
+// where 8 lanes take five to ten.
+template <class MD, bool MF, int BC, int W>
+__global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 ? 4 : 2) interp_near(const typename MD::S* __restrict__ Phi,
                                                    const cplx<typename MD::R>* __restrict__ x,
                                                    cplx<typename MD::R>* __restrict__ y,
                                                    const typename MD::R* __restrict__ lam,
@@ -189,8 +198,8 @@ __global__ void __launch_bounds__(256) interp_near(const typename MD::S* __restr
   using C = cplx<R>;
   __shared__ int s_off[kMaxStencil];
   stencil_offsets_smem(s_off, S, P, nx, ny);
-  const int lane = threadIdx.x & 7;
-  const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int lane = threadIdx.x & (W - 1);
+  const int m = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / W);
   const bool live = m < N;
   const int mm = live ? m : N - 1;
   const int b0 = base[mm];
@@ -204,49 +213,106 @@ __global__ void __launch_bounds__(256) interp_near(const typename MD::S* __restr
 #else
   const int Sc = S;
 #endif
-  for (int b = 0; b < nrhs; ++b) {
-    const typename MD::S* Pb = Phi + (long long)b * 4 * Nc;
-    C av = cmake<C>(0, 0), ar = av, an = av, am = av;
-    for (int s = lane; s < Sc; s += 8) {
+  for (int bc = 0; bc < nrhs; bc += BC) {
+    // t: the EFIE's grid part before its factor j; o: the near part and the MFIE's grid part.
+    // fvec = alpha k eta, frho = alpha eta / k, fmf = (1 - alpha) eta scale the weights once for a
+    // chunk of right-hand sides, the sums (t: vector part, tr: charge, om: MFIE) for a single one.
+    C t[BC], o[BC], tr = cmake<C>(0, 0), om = tr;
+#pragma unroll
+    for (int q = 0; q < BC; ++q) t[q] = o[q] = cmake<C>(0, 0);
+    const typename MD::S* Pb = Phi + (long long)bc * 4 * Nc;
+    for (int s = lane; s < Sc; s += W) {
       const long long node = b0 + (long long)s_off[s];
-      const C px = MD::get(Pb[node]), py = MD::get(Pb[Nc + node]), pz = MD::get(Pb[2 * Nc + node]),
-              pr = MD::get(Pb[3 * Nc + node]);
-      const R wx = lm[s], wy = lm[S + s], wz = lm[2 * S + s], wr = lm[3 * S + s];
-      av.x += wx * px.x + wy * py.x + wz * pz.x;
-      av.y += wx * px.y + wy * py.y + wz * pz.y;
-      ar.x += wr * pr.x;
-      ar.y += wr * pr.y;
+      R wx = lm[s], wy = lm[S + s], wz = lm[2 * S + s], wr = lm[3 * S + s], mx = 0, my = 0, mz = 0;
       if constexpr (MF) {
-        const R mx = wm[s], my = wm[S + s], mz = wm[2 * S + s];
-        am.x += mx * px.x + my * py.x + mz * pz.x;
-        am.y += mx * px.y + my * py.y + mz * pz.y;
+        mx = wm[s];
+        my = wm[S + s];
+        mz = wm[2 * S + s];
+      }
+      if constexpr (BC > 1) {
+        wx *= fvec;
+        wy *= fvec;
+        wz *= fvec;
+        wr *= -frho;
+        mx *= -fmf;
+        my *= -fmf;
+        mz *= -fmf;
+      }
+#pragma unroll
+      for (int q = 0; q < BC; ++q) {
+        if (BC > 1 && bc + q >= nrhs) break;
+        const typename MD::S* Pq = Pb + (long long)q * 4 * Nc;
+        const C px = MD::get(Pq[node]), py = MD::get(Pq[Nc + node]), pz = MD::get(Pq[2 * Nc + node]),
+                pr = MD::get(Pq[3 * Nc + node]);
+        C& r = BC > 1 ? t[q] : tr;
+        C& f = BC > 1 ? o[q] : om;
+        t[q].x += wx * px.x + wy * py.x + wz * pz.x;
+        t[q].y += wx * px.y + wy * py.y + wz * pz.y;
+        r.x += wr * pr.x;
+        r.y += wr * pr.y;
+        if constexpr (MF) {
+          f.x += mx * px.x + my * py.x + mz * pz.x;
+          f.y += mx * px.y + my * py.y + mz * pz.y;
+        }
       }
     }
-    const C* xb = x + (long long)b * N;
-    for (int e = r0 + lane; e < r1; e += 8) {
-      const C v = nval[e], xv = xb[ncol[e]];
-      an.x += v.x * xv.x - v.y * xv.y;
-      an.y += v.x * xv.y + v.y * xv.x;
+    if constexpr (BC == 1) {
+      t[0].x = fvec * t[0].x - frho * tr.x;
+      t[0].y = fvec * t[0].y - frho * tr.y;
+      if constexpr (MF) {
+        o[0].x -= fmf * om.x;
+        o[0].y -= fmf * om.y;
+      }
     }
-    // grid part: j (fvec av - frho ar) - fmf am  with fvec = alpha k eta,
-    // frho = alpha eta / k, fmf = (1 - alpha) eta (am: the MFIE weights' sum)
-    C t;
-    t.x = fvec * av.x - frho * ar.x;
-    t.y = fvec * av.y - frho * ar.y;
-    C out;
-    out.x = an.x - t.y;
-    out.y = an.y + t.x;
-    if constexpr (MF) {
-      out.x -= fmf * am.x;
-      out.y -= fmf * am.y;
+    const C* xb = x + (long long)bc * N;
+#pragma unroll 2
+    for (int e = r0 + lane; e < r1; e += W) {
+      const C v = nval[e];
+      const C* xc = xb + ncol[e];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) {
+        if (BC > 1 && bc + q >= nrhs) break;
+        const C xv = xc[(long long)q * N];
+        o[q].x += v.x * xv.x - v.y * xv.y;
+        o[q].y += v.x * xv.y + v.y * xv.x;
+      }
     }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-      out.x += __shfl_xor_sync(0xffffffffu, out.x, o, 8);
-      out.y += __shfl_xor_sync(0xffffffffu, out.y, o, 8);
+    for (int q = 0; q < BC; ++q) {
+      C out;
+      out.x = o[q].x - t[q].y;
+      out.y = o[q].y + t[q].x;
+#pragma unroll
+      for (int d = W / 2; d > 0; d >>= 1) {
+        out.x += __shfl_xor_sync(0xffffffffu, out.x, d, W);
+        out.y += __shfl_xor_sync(0xffffffffu, out.y, d, W);
+      }
+      if (live && lane == 0 && bc + q < nrhs) y[(long long)(bc + q) * N + m] = out;
     }
-    if (live && lane == 0) y[(long long)b * N + m] = out;
   }
+}
+
+// Calls f(MFIE weights or not, right-hand sides at a time, lanes per basis function) with the
+// interpolation kernels' choices as types: a warp per basis function for N below `small`.  For
+// complex64 that is up to a quarter of the GPU's threads at 8 lanes (7,680 unknowns, 8 right-hand
+// sides: 45 -> 41 us); the 16-byte types pay for the longer reduction, so only a body too small for the
+// GPU takes it (225 unknowns, float-float: 10.3 -> 8.4 us; 14,520: 36 -> 54 us; FP64, 1,470
+// unknowns: 29 -> 21 us; 3,816: 25 -> 30 us).
+constexpr long long kSmallInterp32 = 152LL * 1024 / 16, kSmallInterp64 = 152LL * 1024 / 64;
+template <class F> static void interp_shape(bool mf, int nrhs, bool warp, F&& f) {
+  const auto lanes = [&](auto m, auto bc) {
+    if (warp)
+      f(m, bc, std::integral_constant<int, 32>{});
+    else
+      f(m, bc, std::integral_constant<int, 8>{});
+  };
+  const auto rhs = [&](auto m) {
+    if (nrhs == 1) lanes(m, std::integral_constant<int, 1>{});
+    else if (nrhs == 2) lanes(m, std::integral_constant<int, 2>{});
+    else lanes(m, std::integral_constant<int, 4>{});
+  };
+  if (mf) rhs(std::true_type{});
+  else rhs(std::false_type{});
 }
 
 // out[c][r] = in[r][c] for an R x Cn row-major matrix (32 x 32 tiles through
@@ -671,8 +737,9 @@ __global__ void __launch_bounds__(256) proj_gather_ff(const float4* __restrict__
   }
 }
 
-// Interpolation + near correction: 8 lanes per basis function, as interp_near.
-template <bool MF>
+// Interpolation + near correction: W lanes per basis function, one right-hand side at a time (two
+// at a time take 98 registers and leave half the warps: 36 -> 46 us for 14,520 unknowns, CFIE).
+template <bool MF, int W>
 __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__ Phi, const float4* __restrict__ x,
                                                       double2* __restrict__ y, const float2* __restrict__ lam,
                                                       const int32_t* __restrict__ base, const int32_t* __restrict__ nptr,
@@ -682,8 +749,8 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
                                                       const float2* __restrict__ lamM, float2 fmf) {
   __shared__ int s_off[kMaxStencil];
   stencil_offsets_smem(s_off, S, P, nx, ny);
-  const int lane = threadIdx.x & 7;
-  const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int lane = threadIdx.x & (W - 1);
+  const int m = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / W);
   const bool live = m < N;
   const int mm = live ? m : N - 1;
   const int b0 = base[mm];
@@ -700,9 +767,9 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
   const cff2 kv = cff2_both(ffv(fvec.x, fvec.y)), kr = cff2_both(ffv(-frho.x, -frho.y)),
              km = cff2_both(ffv(-fmf.x, -fmf.y));
   for (int b = 0; b < nrhs; ++b) {
-    const float4* Pb = Phi + (long long)b * 4 * Nc;
     cff2 av = cff2_zero(), ar = av, an = av, am = av;
-    for (int s = lane; s < Sc; s += 8) {
+    const float4* Pb = Phi + (long long)b * 4 * Nc;
+    for (int s = lane; s < Sc; s += W) {
       const long long node = b0 + (long long)s_off[s];
       const cff2 px = cff2_ld(Pb[node]), py = cff2_ld(Pb[Nc + node]), pz = cff2_ld(Pb[2 * Nc + node]),
                  pr = cff2_ld(Pb[3 * Nc + node]);
@@ -719,16 +786,24 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
       }
     }
     const float4* xb = x + (long long)b * N;
-    for (int e = r0 + lane; e < r1; e += 8) {
-      const cff2 v = cff2_ld(nval[e]), xv = cff2_ld(xb[ncol[e]]);
-      an = cff2_mad(cff2_re(v), xv, an);
-      an = cff2_mad(cff2_im(v), cff2_times_i(xv), an);
+    // two entries' gathers in flight per lane
+    for (int e = r0 + lane; e < r1; e += 2 * W) {
+      const bool two = e + W < r1;
+      const int c0 = ncol[e], c1 = two ? ncol[e + W] : c0;
+      const cff2 v0 = cff2_ld(nval[e]), v1 = two ? cff2_ld(nval[e + W]) : cff2_zero();
+      const cff2 x0 = cff2_ld(xb[c0]), x1 = cff2_ld(xb[c1]);
+      an = cff2_mad(cff2_re(v0), x0, an);
+      an = cff2_mad(cff2_im(v0), cff2_times_i(x0), an);
+      if (two) {
+        an = cff2_mad(cff2_re(v1), x1, an);
+        an = cff2_mad(cff2_im(v1), cff2_times_i(x1), an);
+      }
     }
     // an + j (fvec av - frho ar) - fmf am
     cff2 out = cff2_add(an, cff2_times_i(cff2_dot2(kv, av, kr, ar)));
     if constexpr (MF) out = cff2_mad(km, am, out);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) out = cff2_add(out, cff2_shfl_xor(out, o, 8));
+    for (int d = W / 2; d > 0; d >>= 1) out = cff2_add(out, cff2_shfl_xor(out, d, W));
     if (live && lane == 0)
       y[(long long)b * N + m] = make_double2((double)out.hi.x + (double)out.lo.x, (double)out.hi.y + (double)out.lo.y);
   }
@@ -790,20 +865,18 @@ static int run_product_ff(aim_ctx* c, const double2* x, double2* y, int nrhs) {
   }
   AIM_TRY(fft_convolve_ff(c, 4 * nrhs));
   {
-    const long long threads = (long long)c->N * 8;
-    const int blocks = (int)((threads + 255) / 256);
     const double fv = c->alpha * c->k * kEta0, fr = c->alpha * kEta0 / c->k, fm = (1.0 - c->alpha) * kEta0;
     const float fvh = (float)fv, frh = (float)fr, fmh = (float)fm;
     const float2 fvec = make_float2(fvh, (float)(fv - (double)fvh)), frho = make_float2(frh, (float)(fr - (double)frh));
     const float2 fmf = make_float2(fmh, (float)(fm - (double)fmh));
-    const auto go = [&](auto mf) {
+    interp_shape(p.lamM != nullptr, 1, c->N < kSmallInterp64, [&](auto mf, auto, auto w) {
+      constexpr int W = decltype(w)::value;
+      const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
       AIM_LAUNCH(c, "interp_near",
-             (interp_near_ff<decltype(mf)::value><<<blocks, 256, 0, c->stream>>>(phi_grid(c, p.grid0, p.grid2), p.xff, y, p.lam, c->base, c->near_ptr,
-                                                                c->near_col, p.near_val, c->N, Nc, c->n[0], c->n[1],
-                                                                nrhs, fvec, frho, c->S, c->M + 1, p.lamM, fmf)));
-    };
-    if (p.lamM) go(std::true_type{}); else go(std::false_type{});
-
+                 (interp_near_ff<decltype(mf)::value, W><<<blocks, 256, 0, c->stream>>>(
+                     phi_grid(c, p.grid0, p.grid2), p.xff, y, p.lam, c->base, c->near_ptr, c->near_col, p.near_val,
+                     c->N, Nc, c->n[0], c->n[1], nrhs, fvec, frho, c->S, c->M + 1, p.lamM, fmf)));
+    });
     AIM_TRY(launch_check(c, "interp_near"));
   }
   return AIM_OK;
@@ -888,8 +961,12 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const int32_t* groups = c->sparse_proj ? c->pgroups : nullptr;
     const auto go = [&](auto bc) {
-      AIM_LAUNCH(c, "proj_gather", (proj_gather<MD, decltype(bc)::value><<<blocks, 256, 0, c->stream>>>(
-                                       x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
+      if (blocks <= 2 * 152)
+        AIM_LAUNCH(c, "proj_gather", (proj_gather<MD, decltype(bc)::value, 2><<<blocks, 256, 0, c->stream>>>(
+                                         x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
+      else
+        AIM_LAUNCH(c, "proj_gather", (proj_gather<MD, decltype(bc)::value, 1><<<blocks, 256, 0, c->stream>>>(
+                                         x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
     };
     if (nrhs == 1) go(std::integral_constant<int, 1>{});
     else if (nrhs == 2) go(std::integral_constant<int, 2>{});
@@ -926,18 +1003,16 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
     return launch_check(c, "interp_near");
   }
   {
-    const long long threads = (long long)c->N * 8;
-    const int blocks = (int)((threads + 255) / 256);
     const R fvec = (R)(c->alpha * c->k * kEta0), frho = (R)(c->alpha * kEta0 / c->k),
             fmf = (R)((1.0 - c->alpha) * kEta0);
-    const auto go = [&](auto mf) {
-    AIM_LAUNCH(c, "interp_near",
-             (interp_near<MI, decltype(mf)::value><<<blocks, 256, 0, c->stream>>>(phi, x, y, lam, c->base, c->near_ptr,
-                                                                 c->near_col, nval, c->N, Nc, c->n[0], c->n[1],
-                                                                 nrhs, fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
-    };
-    if (pd.lamM) go(std::true_type{}); else go(std::false_type{});
-
+    interp_shape(pd.lamM != nullptr, nrhs, c->N < (sizeof(R) == 4 ? kSmallInterp32 : kSmallInterp64), [&](auto mf, auto bc, auto w) {
+      constexpr int W = decltype(w)::value;
+      const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
+      AIM_LAUNCH(c, "interp_near",
+                 (interp_near<MI, decltype(mf)::value, decltype(bc)::value, W><<<blocks, 256, 0, c->stream>>>(
+                     phi, x, y, lam, c->base, c->near_ptr, c->near_col, nval, c->N, Nc, c->n[0], c->n[1], nrhs, fvec,
+                     frho, c->S, c->M + 1, pd.lamM, fmf)));
+    });
     AIM_TRY(launch_check(c, "interp_near"));
   }
   return AIM_OK;
@@ -1051,7 +1126,7 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
     const long long ntask = (Nc + 7) / 8;
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const auto go = [&](auto bc) {
-      AIM_LAUNCH(c, "proj_gather", (proj_gather<M32, decltype(bc)::value><<<blocks, 256, 0, c->stream>>>(
+      AIM_LAUNCH(c, "proj_gather", (proj_gather<M32, decltype(bc)::value, 1><<<blocks, 256, 0, c->stream>>>(
                                        x, g0, c->pnode_ptr, c->pnode_m, c->p32.pnode_w, c->N, Nc, nrhs, nullptr,
                                        ntask)));
     };
@@ -1062,18 +1137,16 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
   }
   AIM_TRY(fft_convolve_c64_bufs(c, 4 * nrhs, g0, g1, g2));
   {
-    const long long threads = (long long)c->N * 8;
-    const int blocks = (int)((threads + 255) / 256);
     const float fvec = (float)(c->alpha * c->k * kEta0), frho = (float)(c->alpha * kEta0 / c->k),
                 fmf = (float)((1.0 - c->alpha) * kEta0);
-    const auto go = [&](auto mf) {
-    AIM_LAUNCH(c, "interp_near",
-             (interp_near<M32, decltype(mf)::value><<<blocks, 256, 0, c->stream>>>(g0, x, y, c->p32.lam, c->base, c->near_ptr,
-                                                                  c->near_col, c->p32.near_val, c->N, Nc,
-                                                                  c->n[0], c->n[1], nrhs, fvec, frho, c->S, c->M + 1, c->p32.lamM, fmf)));
-    };
-    if (c->p32.lamM) go(std::true_type{}); else go(std::false_type{});
-
+    interp_shape(c->p32.lamM != nullptr, nrhs, c->N < kSmallInterp32, [&](auto mf, auto bc, auto w) {
+      constexpr int W = decltype(w)::value;
+      const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
+      AIM_LAUNCH(c, "interp_near",
+                 (interp_near<M32, decltype(mf)::value, decltype(bc)::value, W><<<blocks, 256, 0, c->stream>>>(
+                     g0, x, y, c->p32.lam, c->base, c->near_ptr, c->near_col, c->p32.near_val, c->N, Nc, c->n[0],
+                     c->n[1], nrhs, fvec, frho, c->S, c->M + 1, c->p32.lamM, fmf)));
+    });
     AIM_TRY(launch_check(c, "interp_near"));
   }
 #ifdef AIM_CHECK

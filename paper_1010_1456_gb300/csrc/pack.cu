@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.h"
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(256) proj_pack(const float2* __restrict__ x, f
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int c = 0; c < 4; ++c) a[q][c] = make_float2(0.f, 0.f);
+#pragma unroll 2
       for (int e = e0 + lane; e < e1; e += 4) {
         const float4 w = reinterpret_cast<const float4*>(d.pw)[e];
         const float2* xc = x + (long long)(d.b0 + bc) * ldx + d.pm[e];
@@ -132,10 +134,11 @@ __global__ void __launch_bounds__(256) proj_pack(const float2* __restrict__ x, f
   }
 }
 
-// Interpolation + near correction, 8 lanes per basis function of any
-// instance (the 8 lanes of a group share one instance, the groups of a warp
-// may not, so the reductions use the group's own lane mask), then the
-// padding of every packed row written as zero.
+// Interpolation + near correction, W lanes per basis function of any instance
+// (they share one instance; the groups of a warp may not, so the reductions
+// use the group's own lane mask), BC right-hand sides at a time (as
+// interp_near), then the padding of every packed row written as zero.
+template <int BC, int W>
 __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Phi, const float2* __restrict__ x,
                                                    float2* __restrict__ y, const PackInst* __restrict__ inst,
                                                    const int32_t* __restrict__ row0, int K, long long rows, int ldx,
@@ -147,9 +150,9 @@ __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Ph
     s_off[s] = (kk * nyp + j) * nxp + ii;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 7;
-  const unsigned gmask = 0xffu << (threadIdx.x & 24);
-  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int lane = threadIdx.x & (W - 1);
+  const unsigned gmask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1) << (threadIdx.x & (32 - W));
+  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / W;
   if (r < rows) {
     int lo = 0, hi = K - 1;  // instance i with row0[i] <= r < row0[i + 1]
     while (lo < hi) {
@@ -161,6 +164,7 @@ __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Ph
     const int bs = d.base[m];
     const float* lm = d.lam + (long long)m * 4 * S;
     const float* wm = d.lamM ? d.lamM + (long long)m * 3 * S : nullptr;
+    const float fvec = d.fvec, frho = d.frho, fmf = d.fmf;
     const int r0 = d.nptr[m];
     int r1 = d.nptr[m + 1];
 #ifdef AIM_CHECK
@@ -169,40 +173,58 @@ __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Ph
 #else
     const int Sc = S;
 #endif
-    for (int b = 0; b < d.nrhs; ++b) {
-      const long long g = d.b0 + b;
+    for (int bc = 0; bc < d.nrhs; bc += BC) {
+      const int nb = min(BC, d.nrhs - bc);
+      const long long g = d.b0 + bc;
       const float2* Pb = Phi + g * 4 * Ncp;
-      float2 av = make_float2(0.f, 0.f), ar = av, an = av, am = av;
-      for (int s = lane; s < Sc; s += 8) {
+      float2 t[BC], o[BC];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) t[q] = o[q] = make_float2(0.f, 0.f);
+      for (int s = lane; s < Sc; s += W) {
         const long long node = bs + (long long)s_off[s];
-        const float2 px = Pb[node], py = Pb[Ncp + node], pz = Pb[2 * Ncp + node], pr = Pb[3 * Ncp + node];
-        const float wx = lm[s], wy = lm[S + s], wz = lm[2 * S + s], wr = lm[3 * S + s];
-        av.x += wx * px.x + wy * py.x + wz * pz.x;
-        av.y += wx * px.y + wy * py.y + wz * pz.y;
-        ar.x += wr * pr.x;
-        ar.y += wr * pr.y;
+        const float wx = fvec * lm[s], wy = fvec * lm[S + s], wz = fvec * lm[2 * S + s], wr = -frho * lm[3 * S + s];
+        float mx = 0.f, my = 0.f, mz = 0.f;
         if (wm) {
-          const float mx = wm[s], my = wm[S + s], mz = wm[2 * S + s];
-          am.x += mx * px.x + my * py.x + mz * pz.x;
-          am.y += mx * px.y + my * py.y + mz * pz.y;
+          mx = -fmf * wm[s];
+          my = -fmf * wm[S + s];
+          mz = -fmf * wm[2 * S + s];
+        }
+#pragma unroll
+        for (int q = 0; q < BC; ++q) {
+          if (q >= nb) break;
+          const float2* Pq = Pb + (long long)q * 4 * Ncp;
+          const float2 px = Pq[node], py = Pq[Ncp + node], pz = Pq[2 * Ncp + node], pr = Pq[3 * Ncp + node];
+          t[q].x += wx * px.x + wy * py.x + wz * pz.x + wr * pr.x;
+          t[q].y += wx * px.y + wy * py.y + wz * pz.y + wr * pr.y;
+          if (wm) {
+            o[q].x += mx * px.x + my * py.x + mz * pz.x;
+            o[q].y += mx * px.y + my * py.y + mz * pz.y;
+          }
         }
       }
       const float2* xb = x + g * ldx;
-      for (int e = r0 + lane; e < r1; e += 8) {
-        const float2 v = d.nval[e], xv = xb[d.ncol[e]];
-        an.x += v.x * xv.x - v.y * xv.y;
-        an.y += v.x * xv.y + v.y * xv.x;
-      }
-      // j (fvec av - frho ar) - fmf am + near
-      float2 out;
-      out.x = an.x - (d.fvec * av.y - d.frho * ar.y) - d.fmf * am.x;
-      out.y = an.y + (d.fvec * av.x - d.frho * ar.x) - d.fmf * am.y;
+#pragma unroll 2
+      for (int e = r0 + lane; e < r1; e += W) {
+        const float2 v = d.nval[e];
+        const float2* xc = xb + d.ncol[e];
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        out.x += __shfl_xor_sync(gmask, out.x, o, 8);
-        out.y += __shfl_xor_sync(gmask, out.y, o, 8);
+        for (int q = 0; q < BC; ++q) {
+          if (q >= nb) break;
+          const float2 xv = xc[(long long)q * ldx];
+          o[q].x += v.x * xv.x - v.y * xv.y;
+          o[q].y += v.x * xv.y + v.y * xv.x;
+        }
       }
-      if (lane == 0) y[g * ldx + m] = out;
+#pragma unroll
+      for (int q = 0; q < BC; ++q) {
+        float2 out = make_float2(o[q].x - t[q].y, o[q].y + t[q].x);
+#pragma unroll
+        for (int h = W / 2; h > 0; h >>= 1) {
+          out.x += __shfl_xor_sync(gmask, out.x, h, W);
+          out.y += __shfl_xor_sync(gmask, out.y, h, W);
+        }
+        if (lane == 0 && q < nb) y[(g + q) * ldx + m] = out;
+      }
     }
   }
   const long long nth = (long long)gridDim.x * blockDim.x;
@@ -235,12 +257,17 @@ static int pack_c64(aim_pack* P, const float2* x, float2* y) {
   }
   AIM_TRY(fft_convolve_c64(c, 4 * P->B));
   {
-    const long long threads = P->rows * 8;
-    const int blocks = (int)std::max<long long>(1, (threads + 255) / 256);
-    AIM_LAUNCH(c, "interp_pack",
-               (interp_pack<<<blocks, 256, 0, c->stream>>>(phi_grid(c, c->p32.grid0, c->p32.grid2), x, y, P->d_inst,
-                                                           P->d_row0, P->K, P->rows, P->ld, c->n[0], c->n[1], Ncp,
-                                                           c->S, c->M + 1, P->d_rhsN, P->B)));
+    // a warp per basis function while 8 lanes would leave three quarters of the GPU's threads unused
+    const auto go = [&](auto w) {
+      constexpr int W = decltype(w)::value;
+      const unsigned blocks = (unsigned)std::max<long long>(1, (P->rows * W + 255) / 256);
+      AIM_LAUNCH(c, "interp_pack",
+                 (interp_pack<4, W><<<blocks, 256, 0, c->stream>>>(phi_grid(c, c->p32.grid0, c->p32.grid2), x, y,
+                                                                   P->d_inst, P->d_row0, P->K, P->rows, P->ld, c->n[0],
+                                                                   c->n[1], Ncp, c->S, c->M + 1, P->d_rhsN, P->B)));
+    };
+    if (P->rows * 32 < 152LL * 1024) go(std::integral_constant<int, 32>{});
+    else go(std::integral_constant<int, 8>{});
     AIM_TRY(launch_check(c, "interp_pack"));
   }
   return AIM_OK;
