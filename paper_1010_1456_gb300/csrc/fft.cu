@@ -241,6 +241,7 @@ template <class P, bool INV, class O>
 __global__ void __launch_bounds__(256) fft_strided(const typename P::S* __restrict__ in, O* __restrict__ out,
                                                    StridedArgs a, const FftPlan* __restrict__ plan,
                                                    const typename P::S* __restrict__ tw) {
+  pdl_begin();
   using S = typename P::S;
   constexpr int TX = P::kTX;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -282,6 +283,7 @@ struct XArgs {
 template <class P, int MODE>
 __global__ void __launch_bounds__(256) fft_x(typename P::S* __restrict__ buf, XArgs a, const FftPlan* __restrict__ plan,
                                              const typename P::S* __restrict__ ghat, const typename P::S* __restrict__ tw) {
+  pdl_begin();
   using S = typename P::S;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FftPlan& pl = *plan;
@@ -334,7 +336,7 @@ static int launch_strided(aim_ctx* c, const char* name, const typename P::S* in,
       cudaFuncSetAttribute(fft_strided<P, INV, O>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   AIM_CUDA_TRY(attr);
   dim3 grid((a.X + TX - 1) / TX, a.A, G);
-  AIM_LAUNCH(c, name, fft_strided<P, INV, O><<<grid, 256, sm, c->stream>>>(in, out, a, plan_dev, tw));
+  AIM_LAUNCH(c, name, launch_pdl(!std::is_same<P, P64>::value, fft_strided<P, INV, O>, grid, 256, sm, c->stream, in, out, a, plan_dev, tw));
   return launch_check(c, name);
 }
 
@@ -357,7 +359,7 @@ static int launch_x(aim_ctx* c, const char* name, typename P::S* buf, XArgs a, c
       cudaFuncSetAttribute(fft_x<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   AIM_CUDA_TRY(attr);
   dim3 grid(a.rows_y, a.rows_z);
-  AIM_LAUNCH(c, name, fft_x<P, MODE><<<grid, 256, sm, c->stream>>>(buf, a, plan_dev, ghat, tw));
+  AIM_LAUNCH(c, name, launch_pdl(!std::is_same<P, P64>::value, fft_x<P, MODE>, grid, 256, sm, c->stream, buf, a, plan_dev, ghat, tw));
   return launch_check(c, name);
 }
 

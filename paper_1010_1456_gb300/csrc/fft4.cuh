@@ -134,6 +134,7 @@ template <class P, bool INV, int L1, int L2, bool PRUNED>
 __global__ void __launch_bounds__(strided_threads<P, L1, L2>(), strided_min_blocks<P, L1, L2>())
     fft4_strided(const typename P::S* __restrict__ in, typename P::S* __restrict__ out, StridedArgs4 a,
                  const typename P::S* __restrict__ twL, int AY) {
+  pdl_begin();
   using S = typename P::S;
   using T = typename P::T;
   constexpr int L = L1 * L2, TX = strided_tx<P, L>(), RP = strided_row<P, L1, L2>();
@@ -209,6 +210,7 @@ template <class P, int L1, int L2>
 __global__ void __launch_bounds__(x_threads<P>(), x_min_blocks<P, L1, L2>()) fft4_x(typename P::S* __restrict__ buf, XArgs4 a,
                                               const typename P::S* __restrict__ ghat,
                                               const typename P::S* __restrict__ twL) {
+  pdl_begin();
   using S = typename P::S;
   using T = typename P::T;
   constexpr int L = L1 * L2;

@@ -32,7 +32,7 @@ int launch_strided4(aim_ctx* c, const char* name, const S* in, S* out, const Str
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   AIM_CUDA_TRY(attr);
   dim3 grid((unsigned)xt, (a.A + AY - 1) / AY, G);
-  AIM_LAUNCH(c, name, (kern<<<grid, threads, sm, c->stream>>>(in, out, a, tw, AY)));
+  AIM_LAUNCH(c, name, (launch_pdl(!std::is_same<Pol, P64>::value, kern, grid, threads, sm, c->stream, in, out, a, tw, AY)));
   return launch_check(c, name);
 }
 
@@ -111,7 +111,7 @@ int launch_x4(aim_ctx* c, const char* name, S* buf, XArgs4 a, const S* ghat, con
       cudaFuncSetAttribute(fft4_x<Pol, L1, L2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   AIM_CUDA_TRY(attr);
   dim3 grid((a.Ly + RY - 1) / RY, a.Lz, (a.G + GB - 1) / GB);
-  AIM_LAUNCH(c, name, (fft4_x<Pol, L1, L2><<<grid, nthreads, sm, c->stream>>>(buf, a, ghat, tw)));
+  AIM_LAUNCH(c, name, (launch_pdl(!std::is_same<Pol, P64>::value, fft4_x<Pol, L1, L2>, grid, nthreads, sm, c->stream, buf, a, ghat, tw)));
   return launch_check(c, name);
 }
 }  // namespace

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(256) proj_gather(const cplx<typename MD::R>* _
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ mm,
                                                    const typename MD::R* __restrict__ w, int N, long long Nc, int nrhs,
                                                    const int32_t* __restrict__ groups, long long ntask) {
+  pdl_begin();
   using R = typename MD::R;
   using C = cplx<R>;
   const int lane = threadIdx.x & 3;
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 ? 4 : 2) inte
                                                    int nx, int ny, int nrhs, typename MD::R fvec, typename MD::R frho,
                                                    int S, int P, const typename MD::R* __restrict__ lamM,
                                                    typename MD::R fmf) {
+  pdl_begin();
   using R = typename MD::R;
   using C = cplx<R>;
   __shared__ int s_off[kMaxStencil];
@@ -319,6 +321,7 @@ template <class F> static void interp_shape(bool mf, int nrhs, bool warp, F&& f)
 // shared memory, so both the reads and the writes are coalesced).
 template <class E>
 __global__ void __launch_bounds__(256) k_transpose(const E* __restrict__ in, E* __restrict__ out, int R, long long Cn) {
+  pdl_begin();
   __shared__ E t[32][33];
   const long long c0 = blockIdx.x * 32LL;
   const int r0 = blockIdx.y * 32;
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(256) k_transpose(const E* __restrict__ in, E* 
 template <class E>
 static int transpose(aim_ctx* c, const char* name, const E* in, E* out, int R, long long Cn) {
   dim3 grid((unsigned)((Cn + 31) / 32), (unsigned)((R + 31) / 32));
-  AIM_LAUNCH(c, name, (k_transpose<E><<<grid, dim3(32, 8), 0, c->stream>>>(in, out, R, Cn)));
+  AIM_LAUNCH(c, name, (launch_pdl(sizeof(E) <= 8, k_transpose<E>, grid, dim3(32, 8), 0, c->stream, in, out, R, Cn)));
   return launch_check(c, name);
 }
 
@@ -433,6 +436,7 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
                                                        long long Nc, int nx, int ny, int B, typename MI::R fvec,
                                                        typename MI::R frho, int S, int P,
                                                        const typename MI::R* __restrict__ lamM, typename MI::R fmf) {
+  pdl_begin();
   using R = typename MI::R;
   using C = cplx<R>;
   constexpr int G = kNearGroup;
@@ -574,6 +578,7 @@ __global__ void __launch_bounds__(256) proj_gather_rhs(const cplx<typename MD::R
                                                        const int32_t* __restrict__ mm,
                                                        const typename MD::R* __restrict__ w, long long Nc, int B,
                                                        int ldx, int N) {
+  pdl_begin();
   using R = typename MD::R;
   using C = cplx<R>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -652,6 +657,7 @@ __global__ void k_real_to_ff(const double* __restrict__ in, float2* __restrict__
   }
 }
 __global__ void k_cplx_to_ff(const double2* __restrict__ in, float4* __restrict__ out, long long n) {
+  pdl_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const ff re = ff_from_double(in[i].x), im = ff_from_double(in[i].y);
     out[i] = make_float4(re.hi, im.hi, re.lo, im.lo);
@@ -676,6 +682,7 @@ __global__ void __launch_bounds__(256) proj_gather_ff(const float4* __restrict__
                                                       const int32_t* __restrict__ ptr, const int32_t* __restrict__ mm,
                                                       const float4* __restrict__ w, int N, long long Nc, int nrhs,
                                                       const int32_t* __restrict__ groups, long long ntask) {
+  pdl_begin();
   const int lane = threadIdx.x & 3;
   const ProjTasks tasks{groups, ntask, Nc, (int)((threadIdx.x & 31) >> 2)};
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -747,6 +754,7 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
                                                       const float4* __restrict__ nval, int N, long long Nc, int nx,
                                                       int ny, int nrhs, float2 fvec, float2 frho, int S, int P,
                                                       const float2* __restrict__ lamM, float2 fmf) {
+  pdl_begin();
   __shared__ int s_off[kMaxStencil];
   stencil_offsets_smem(s_off, S, P, nx, ny);
   const int lane = threadIdx.x & (W - 1);
@@ -832,7 +840,7 @@ static int ensure_ff_arrays(aim_ctx* c) {
     AIM_TRY(launch_check(c, "weights_to_ff"));
   }
   if (c->nnz > 0) {
-    AIM_LAUNCH(c, "weights_to_ff", (k_cplx_to_ff<<<blocks, 256, 0, c->stream>>>(c->p64.near_val, p.near_val, c->nnz)));
+    AIM_LAUNCH(c, "weights_to_ff", (launch_pdl(true, k_cplx_to_ff, blocks, 256, 0, c->stream, c->p64.near_val, p.near_val, c->nnz)));
     AIM_TRY(launch_check(c, "weights_to_ff"));
   }
   return AIM_OK;
@@ -845,7 +853,7 @@ static int run_product_ff(aim_ctx* c, const double2* x, double2* y, int nrhs) {
   const long long nx_ = (long long)nrhs * c->N;
   {
     const int blocks = (int)std::min<long long>((nx_ + 255) / 256, 152LL * 8);
-    AIM_LAUNCH(c, "x_to_ff", (k_cplx_to_ff<<<blocks, 256, 0, c->stream>>>(x, p.xff, nx_)));
+    AIM_LAUNCH(c, "x_to_ff", (launch_pdl(true, k_cplx_to_ff, blocks, 256, 0, c->stream, x, p.xff, nx_)));
     AIM_TRY(launch_check(c, "x_to_ff"));
   }
   {
@@ -854,7 +862,7 @@ static int run_product_ff(aim_ctx* c, const double2* x, double2* y, int nrhs) {
     const int32_t* groups = c->sparse_proj ? c->pgroups : nullptr;
     const auto go = [&](auto bc) {
       AIM_LAUNCH(c, "proj_gather",
-                 (proj_gather_ff<decltype(bc)::value><<<blocks, 256, 0, c->stream>>>(p.xff, p.grid0, c->pnode_ptr,
+                 (launch_pdl(true, proj_gather_ff<decltype(bc)::value>, blocks, 256, 0, c->stream, p.xff, p.grid0, c->pnode_ptr,
                                                                                       c->pnode_m, p.pnode_w, c->N, Nc,
                                                                                       nrhs, groups, ntask)));
     };
@@ -873,7 +881,7 @@ static int run_product_ff(aim_ctx* c, const double2* x, double2* y, int nrhs) {
       constexpr int W = decltype(w)::value;
       const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
       AIM_LAUNCH(c, "interp_near",
-                 (interp_near_ff<decltype(mf)::value, W><<<blocks, 256, 0, c->stream>>>(
+                 (launch_pdl(true, interp_near_ff<decltype(mf)::value, W>, blocks, 256, 0, c->stream, 
                      phi_grid(c, p.grid0, p.grid2), p.xff, y, p.lam, c->base, c->near_ptr, c->near_col, p.near_val,
                      c->N, Nc, c->n[0], c->n[1], nrhs, fvec, frho, c->S, c->M + 1, p.lamM, fmf)));
     });
@@ -947,11 +955,11 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
       const cplx<R>* xs = pd.xT + b0;
       typename MD::S* qd = grid0 + (long long)b0 * 4 * Nc;
       if (nb == 64 && nrhs % 2 == 0)  // two per lane: 16-byte loads need an even row stride
-        AIM_LAUNCH(c, "proj_gather", (proj_gather_rhs<MD, 2><<<blocks, 256, sm, c->stream>>>(xs, qd, c->pnode_ptr,
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather_rhs<MD, 2>, blocks, 256, sm, c->stream, xs, qd, c->pnode_ptr,
                                                                                             c->pnode_m, pw, Nc, nb,
                                                                                             nrhs, c->N)));
       else
-        AIM_LAUNCH(c, "proj_gather", (proj_gather_rhs<MD, 1><<<blocks, 256, sm, c->stream>>>(xs, qd, c->pnode_ptr,
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather_rhs<MD, 1>, blocks, 256, sm, c->stream, xs, qd, c->pnode_ptr,
                                                                                             c->pnode_m, pw, Nc, nb,
                                                                                             nrhs, c->N)));
       AIM_TRY(launch_check(c, "proj_gather"));
@@ -962,10 +970,10 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
     const int32_t* groups = c->sparse_proj ? c->pgroups : nullptr;
     const auto go = [&](auto bc) {
       if (blocks <= 2 * 152)
-        AIM_LAUNCH(c, "proj_gather", (proj_gather<MD, decltype(bc)::value, 2><<<blocks, 256, 0, c->stream>>>(
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, decltype(bc)::value, 2>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
       else
-        AIM_LAUNCH(c, "proj_gather", (proj_gather<MD, decltype(bc)::value, 1><<<blocks, 256, 0, c->stream>>>(
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, decltype(bc)::value, 1>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
     };
     if (nrhs == 1) go(std::integral_constant<int, 1>{});
@@ -989,7 +997,7 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
                                                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       AIM_CUDA_TRY(attr);
       AIM_LAUNCH(c, "interp_near",
-                 (interp_near_grp<MI, RL, MF><<<blocks, 256, sm, c->stream>>>(
+                 (launch_pdl(sizeof(typename MI::R) == 4, interp_near_grp<MI, RL, MF>, blocks, 256, sm, c->stream, 
                      pd.phiT, pd.xT, y, lam, c->base, c->ngrp_ptr, c->ngrp_col, pd.ngrp_val, c->N, Nc, c->n[0],
                      c->n[1], nrhs, fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
       return AIM_OK;
@@ -1009,7 +1017,7 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
       constexpr int W = decltype(w)::value;
       const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
       AIM_LAUNCH(c, "interp_near",
-                 (interp_near<MI, decltype(mf)::value, decltype(bc)::value, W><<<blocks, 256, 0, c->stream>>>(
+                 (launch_pdl(sizeof(typename MI::R) == 4, interp_near<MI, decltype(mf)::value, decltype(bc)::value, W>, blocks, 256, 0, c->stream, 
                      phi, x, y, lam, c->base, c->near_ptr, c->near_col, nval, c->N, Nc, c->n[0], c->n[1], nrhs, fvec,
                      frho, c->S, c->M + 1, pd.lamM, fmf)));
     });
@@ -1094,22 +1102,24 @@ int matvec(aim_ctx* c, const void* x, void* y, int nrhs, int precision) {
 }
 
 __global__ void k_c128_to_c64(const double2* __restrict__ in, float2* __restrict__ out, long long n) {
+  pdl_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 __global__ void k_c64_to_c128(const float2* __restrict__ in, double2* __restrict__ out, long long n) {
+  pdl_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = make_double2((double)in[i].x, (double)in[i].y);
 }
 
 int convert_c128_to_c64(aim_ctx* c, const double2* in, float2* out, int64_t count) {
   int blocks = (int)std::min<long long>((count + 255) / 256, 152LL * 8);
-  AIM_LAUNCH(c, "k_c128_to_c64", k_c128_to_c64<<<blocks, 256, 0, c->stream>>>(in, out, count));
+  AIM_LAUNCH(c, "k_c128_to_c64", launch_pdl(true, k_c128_to_c64, blocks, 256, 0, c->stream, in, out, count));
   return launch_check(c, "c128_to_c64");
 }
 int convert_c64_to_c128(aim_ctx* c, const float2* in, double2* out, int64_t count) {
   int blocks = (int)std::min<long long>((count + 255) / 256, 152LL * 8);
-  AIM_LAUNCH(c, "k_c64_to_c128", k_c64_to_c128<<<blocks, 256, 0, c->stream>>>(in, out, count));
+  AIM_LAUNCH(c, "k_c64_to_c128", launch_pdl(true, k_c64_to_c128, blocks, 256, 0, c->stream, in, out, count));
   return launch_check(c, "c64_to_c128");
 }
 
@@ -1126,7 +1136,7 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
     const long long ntask = (Nc + 7) / 8;
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const auto go = [&](auto bc) {
-      AIM_LAUNCH(c, "proj_gather", (proj_gather<M32, decltype(bc)::value, 1><<<blocks, 256, 0, c->stream>>>(
+      AIM_LAUNCH(c, "proj_gather", (launch_pdl(true, proj_gather<M32, decltype(bc)::value, 1>, blocks, 256, 0, c->stream, 
                                        x, g0, c->pnode_ptr, c->pnode_m, c->p32.pnode_w, c->N, Nc, nrhs, nullptr,
                                        ntask)));
     };
@@ -1143,7 +1153,7 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
       constexpr int W = decltype(w)::value;
       const unsigned blocks = (unsigned)(((long long)c->N * W + 255) / 256);
       AIM_LAUNCH(c, "interp_near",
-                 (interp_near<M32, decltype(mf)::value, decltype(bc)::value, W><<<blocks, 256, 0, c->stream>>>(
+                 (launch_pdl(true, interp_near<M32, decltype(mf)::value, decltype(bc)::value, W>, blocks, 256, 0, c->stream, 
                      g0, x, y, c->p32.lam, c->base, c->near_ptr, c->near_col, c->p32.near_val, c->N, Nc, c->n[0],
                      c->n[1], nrhs, fvec, frho, c->S, c->M + 1, c->p32.lamM, fmf)));
     });

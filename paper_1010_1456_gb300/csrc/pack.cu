@@ -77,6 +77,7 @@ constexpr int kPackMaxStencil = 216;
 __global__ void __launch_bounds__(256) proj_pack(const float2* __restrict__ x, float2* __restrict__ Q,
                                                  const PackInst* __restrict__ inst, int K, int ldx, int nxp, int nyp,
                                                  long long Ncp, long long ntask) {
+  pdl_begin();
   const int lane = threadIdx.x & 3, slot = (threadIdx.x & 31) >> 2;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < (long long)K * ntask; t += nwarps) {
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Ph
                                                    const int32_t* __restrict__ row0, int K, long long rows, int ldx,
                                                    int nxp, int nyp, long long Ncp, int S, int P,
                                                    const int32_t* __restrict__ rhsN, int B) {
+  pdl_begin();
   __shared__ int s_off[kPackMaxStencil];
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     const int ii = s % P, j = (s / P) % P, kk = s / (P * P);
@@ -251,7 +253,7 @@ static int pack_c64(aim_pack* P, const float2* x, float2* y) {
   {
     const long long ntask = (Ncp + 7) / 8;
     const int blocks = (int)std::min<long long>((P->K * ntask + 7) / 8, 152LL * 16);
-    AIM_LAUNCH(c, "proj_pack", (proj_pack<<<blocks, 256, 0, c->stream>>>(x, c->p32.grid0, P->d_inst, P->K, P->ld,
+    AIM_LAUNCH(c, "proj_pack", (launch_pdl(true, proj_pack, blocks, 256, 0, c->stream, x, c->p32.grid0, P->d_inst, P->K, P->ld,
                                                                          c->n[0], c->n[1], Ncp, ntask)));
     AIM_TRY(launch_check(c, "proj_pack"));
   }
@@ -262,7 +264,7 @@ static int pack_c64(aim_pack* P, const float2* x, float2* y) {
       constexpr int W = decltype(w)::value;
       const unsigned blocks = (unsigned)std::max<long long>(1, (P->rows * W + 255) / 256);
       AIM_LAUNCH(c, "interp_pack",
-                 (interp_pack<4, W><<<blocks, 256, 0, c->stream>>>(phi_grid(c, c->p32.grid0, c->p32.grid2), x, y,
+                 (launch_pdl(true, interp_pack<4, W>, blocks, 256, 0, c->stream, phi_grid(c, c->p32.grid0, c->p32.grid2), x, y,
                                                                    P->d_inst, P->d_row0, P->K, P->rows, P->ld, c->n[0],
                                                                    c->n[1], Ncp, c->S, c->M + 1, P->d_rhsN, P->B)));
     };
