@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256) fft_strided(const typename P::S* __restri
 
 // ------------------------------------------------------------------ x pass
 struct XArgs {
-  int nx;          // samples per row kept (read and written)
+  int nx, px;      // samples per row kept (read and written), row length in memory
   int rows_y;      // Ly
   int rows_z;      // Lz
   int G;           // grids
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(256) fft_x(typename P::S* __restrict__ buf, XA
   S* b0 = gr + L;
   S* b1 = b0 + a.TG * L;
   const int ky = blockIdx.x, kz = blockIdx.y;
-  const long long row = ((long long)kz * a.rows_y + ky) * a.nx;
+  const long long row = ((long long)kz * a.rows_y + ky) * a.px;
   if (MODE == 0) {
     const int iy = min(ky, a.rows_y - ky), iz = min(kz, a.rows_z - kz);
     const S* grow = ghat + ((long long)iz * a.hy + iy) * a.hx;
@@ -403,7 +403,7 @@ static int x_pass(aim_ctx* c, const char* name, typename P::S* buf, XArgs a, con
   const int k = fft_kernel_for(c, policy_index<P>(), 2);
   if (k != AIM_FFT_STOCKHAM) {
     XArgs4 x4{};
-    x4.nx = a.nx; x4.Ly = a.rows_y; x4.Lz = a.rows_z; x4.G = a.G; x4.sG = a.sG; x4.hx = a.hx; x4.hy = a.hy;
+    x4.nx = a.nx; x4.px = a.px; x4.Ly = a.rows_y; x4.Lz = a.rows_z; x4.G = a.G; x4.sG = a.sG; x4.hx = a.hx; x4.hy = a.hy;
     const int rc = Fft4<P>::x(L, c, name, buf, x4, L, ghat, tw, k == AIM_FFT_FOURSTEP_SMALL ? 128 : 256);
     if (rc == 1) return AIM_OK;
     if (rc < 0) return -rc;
@@ -413,47 +413,49 @@ static int x_pass(aim_ctx* c, const char* name, typename P::S* buf, XArgs a, con
 
 template <class P>
 static int convolve(aim_ctx* c, typename P::S* g0, typename P::S* g1, typename P::S* g2, const typename P::S* ghat,
-                    typename P::S* const* tw, int G, typename P::S* phi) {
+                    typename P::S* const* tw, int G, typename P::S* phi, int px) {
   const int nx = c->n[0], ny = c->n[1], nz = c->n[2];
   const int Lx = c->L[0], Ly = c->L[1], Lz = c->L[2];
   const FftPlan* pd = c->plan_dev;
   // A planar grid (Lz = nz = 1) has no z passes: the y passes read and write g0.
   const bool zpass = Lz > 1;
   typename P::S* gz = zpass ? g1 : g0;
-  if (zpass) {  // z forward: g0 [G][nz][ny][nx] -> g1 [G][Lz][ny][nx]
+  // rows of g1 and g2 are px apart, those of g0 and phi nx
+  const int pz = zpass ? px : nx;
+  if (zpass) {  // z forward: g0 [G][nz][ny][nx] -> g1 [G][Lz][ny][px]
     StridedArgs a{};
     a.n_in = nz; a.n_out = Lz; a.X = nx; a.A = ny;
     a.cols = c->colmask;  // empty (x, y) columns read nothing
     a.sG_in = (long long)nz * ny * nx; a.sA_in = nx; a.sP_in = (long long)ny * nx;
-    a.sG_out = (long long)Lz * ny * nx; a.sA_out = nx; a.sP_out = (long long)ny * nx;
+    a.sG_out = (long long)Lz * ny * px; a.sA_out = px; a.sP_out = (long long)ny * px;
     AIM_TRY((strided_pass<P, false>(c, 0, "fft_z_fwd", g0, g1, a, G, pd + 2, Lz, tw[2])));
   }
-  {  // y forward: gz [G][Lz][ny][nx] -> g2 [G][Lz][Ly][nx]
+  {  // y forward: gz [G][Lz][ny][pz] -> g2 [G][Lz][Ly][px]
     StridedArgs a{};
     a.n_in = ny; a.n_out = Ly; a.X = nx; a.A = Lz;
-    a.sG_in = (long long)Lz * ny * nx; a.sA_in = (long long)ny * nx; a.sP_in = nx;
-    a.sG_out = (long long)Lz * Ly * nx; a.sA_out = (long long)Ly * nx; a.sP_out = nx;
+    a.sG_in = (long long)Lz * ny * pz; a.sA_in = (long long)ny * pz; a.sP_in = pz;
+    a.sG_out = (long long)Lz * Ly * px; a.sA_out = (long long)Ly * px; a.sP_out = px;
     AIM_TRY((strided_pass<P, false>(c, 1, "fft_y_fwd", gz, g2, a, G, pd + 1, Ly, tw[1])));
   }
   {  // x: forward, times Ghat, inverse, in place on g2
     XArgs a{};
-    a.nx = nx; a.rows_y = Ly; a.rows_z = Lz; a.G = G;
-    a.sG = (long long)Lz * Ly * nx;
+    a.nx = nx; a.px = px; a.rows_y = Ly; a.rows_z = Lz; a.G = G;
+    a.sG = (long long)Lz * Ly * px;
     a.hx = Lx / 2 + 1; a.hy = Ly / 2 + 1; a.hz = Lz / 2 + 1;
     AIM_TRY((x_pass<P>(c, "fft_x_conv", g2, a, pd + 0, Lx, ghat, tw[0])));
   }
-  {  // y inverse: g2 -> gz [G][Lz][ny][nx]
+  {  // y inverse: g2 -> gz [G][Lz][ny][pz]
     StridedArgs a{};
     a.n_in = Ly; a.n_out = ny; a.X = nx; a.A = Lz;
-    a.sG_in = (long long)Lz * Ly * nx; a.sA_in = (long long)Ly * nx; a.sP_in = nx;
-    a.sG_out = (long long)Lz * ny * nx; a.sA_out = (long long)ny * nx; a.sP_out = nx;
+    a.sG_in = (long long)Lz * Ly * px; a.sA_in = (long long)Ly * px; a.sP_in = px;
+    a.sG_out = (long long)Lz * ny * pz; a.sA_out = (long long)ny * pz; a.sP_out = pz;
     AIM_TRY((strided_pass<P, true>(c, 3, "fft_y_inv", g2, gz, a, G, pd + 1, Ly, tw[1])));
   }
   if (zpass) {  // z inverse: g1 -> phi [G][nz][ny][nx] (g0, or g2 when grid0 keeps the projection's zeros)
     StridedArgs a{};
     a.n_in = Lz; a.n_out = nz; a.X = nx; a.A = ny;
     a.cols = c->colmask;  // columns without a stencil node are never interpolated from
-    a.sG_in = (long long)Lz * ny * nx; a.sA_in = nx; a.sP_in = (long long)ny * nx;
+    a.sG_in = (long long)Lz * ny * px; a.sA_in = px; a.sP_in = (long long)ny * px;
     a.sG_out = (long long)nz * ny * nx; a.sA_out = nx; a.sP_out = (long long)ny * nx;
     AIM_TRY((strided_pass<P, true>(c, 4, "fft_z_inv", g1, phi, a, G, pd + 2, Lz, tw[2])));
   }
@@ -462,15 +464,15 @@ static int convolve(aim_ctx* c, typename P::S* g0, typename P::S* g1, typename P
 
 int fft_convolve_c64(aim_ctx* c, int G) {
   PrecData<float>& p = c->p32;
-  return convolve<P32>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2));
+  return convolve<P32>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2), c->px);
 }
 int fft_convolve_c128(aim_ctx* c, int G) {
   PrecData<double>& p = c->p64;
-  return convolve<P64>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2));
+  return convolve<P64>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2), c->px);
 }
 int fft_convolve_ff(aim_ctx* c, int G) {
   FFData& p = c->pff;
-  return convolve<PFF>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2));
+  return convolve<PFF>(c, p.grid0, p.grid1, p.grid2, p.ghat, p.tw, G, phi_grid(c, p.grid0, p.grid2), c->px);
 }
 
 // ------------------------------------------------------------------ Ghat
@@ -546,7 +548,7 @@ int build_ghat(aim_ctx* c) {
   s.sA_out = (long long)Ly * Lx; s.sP_out = Lx;
   AIM_TRY(pass("ghat_y", b, a, s, 1));
   XArgs x{};
-  x.nx = Lx; x.rows_y = Ly; x.rows_z = Lz; x.G = 1; x.sG = total;
+  x.nx = x.px = Lx; x.rows_y = Ly; x.rows_z = Lz; x.G = 1; x.sG = total;
   x.hx = Lx / 2 + 1; x.hy = Ly / 2 + 1; x.hz = Lz / 2 + 1;
   AIM_TRY((launch_x<P64, 1>(c, "ghat_x", a, x, c->plan_dev + 0, Lx, nullptr, c->p64.tw[0])));
   AIM_LAUNCH(c, "extract_octant",
@@ -564,6 +566,6 @@ namespace aim {
 // Complex64 convolution on caller-provided pass buffers (used by the
 // product variant that allocates nothing; same kernels and launch shapes).
 int fft_convolve_c64_bufs(aim_ctx* c, int G, float2* g0, float2* g1, float2* g2) {
-  return convolve<P32>(c, g0, g1, g2, c->p32.ghat, c->p32.tw, G, g0);
+  return convolve<P32>(c, g0, g1, g2, c->p32.ghat, c->p32.tw, G, g0, c->n[0]);
 }
 }  // namespace aim

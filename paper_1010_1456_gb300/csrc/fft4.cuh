@@ -41,7 +41,8 @@ struct StridedArgs4 {
 };
 
 struct XArgs4 {
-  int nx, Ly, Lz, G;
+  int nx, px;      // samples per row, row length in memory
+  int Ly, Lz, G;
   int RY, TG;      // rows and grids per block at a time
   int GB;          // grids per block in all (blockIdx.z picks them)
   long long sG;    // grid stride (elements)
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(x_threads<P>(), x_min_blocks<P, L1, L2>()) fft
     const int iy = min(ky, a.Ly - ky);
     gr[e] = ghat[((long long)iz * a.hy + iy) * a.hx + min(p, L - p)];
   }
-  const long long row0 = ((long long)kz * a.Ly + ky0) * a.nx;
+  const long long row0 = ((long long)kz * a.Ly + ky0) * a.px;
   const int gbeg = blockIdx.z * a.GB, gend = min(a.G, gbeg + a.GB);
   for (int g0 = gbeg; g0 < gend; g0 += TG) {
     const int ng = min(TG, gend - g0);
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(x_threads<P>(), x_min_blocks<P, L1, L2>()) fft
     for (int u = threadIdx.x; u < np * L2; u += blockDim.x) {
       const int n2 = u % L2, pc = u / L2;
       const int r = pc / ng, gl = pc - r * ng;
-      const S* src = buf + (long long)(g0 + gl) * a.sG + row0 + (long long)r * a.nx;
+      const S* src = buf + (long long)(g0 + gl) * a.sG + row0 + (long long)r * a.px;
       T v[L1];
       static_for<0, H>([&](auto n1) {
         const int p = L2 * decltype(n1)::value + n2;
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(x_threads<P>(), x_min_blocks<P, L1, L2>()) fft
       T v[L1];
       static_for<0, L1>([&](auto k1) { v[k1] = P::ld(z[decltype(k1)::value * RA]); });
       RegDFT<P, L1, true>::run(v);
-      S* dst = buf + (long long)(g0 + gl) * a.sG + row0 + (long long)r * a.nx;
+      S* dst = buf + (long long)(g0 + gl) * a.sG + row0 + (long long)r * a.px;
       static_for<0, H>([&](auto n1) {
         const int p = n2 + L2 * decltype(n1)::value;
         if (p < a.nx) dst[p] = P::st(v[n1]);

@@ -1028,8 +1028,8 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
 
 int ensure_grids(aim_ctx* c, int precision) {
   const long long B = c->max_rhs;
-  const long long nx = c->n[0], ny = c->n[1], nz = c->n[2], Ly = c->L[1], Lz = c->L[2];
-  const long long e0 = B * 4 * nz * ny * nx, e1 = B * 4 * Lz * ny * nx, e2 = B * 4 * Lz * Ly * nx;
+  const long long nx = c->n[0], ny = c->n[1], nz = c->n[2], Ly = c->L[1], Lz = c->L[2], px = c->px;
+  const long long e0 = B * 4 * nz * ny * nx, e1 = B * 4 * Lz * ny * px, e2 = B * 4 * Lz * Ly * px;
   if (precision == AIM_C64) {
     PrecData<float>& p = c->p32;
     if (!p.grid0) {

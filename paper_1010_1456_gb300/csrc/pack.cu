@@ -354,6 +354,7 @@ static int build_pack(aim_pack* P) {
     }
     c->plan[d] = make_plan(c->L[d]);
   }
+  c->px = row_pitch(c->n[0], 0);
   c->k = c0->k;
   c->h = c0->h;
   c->M = c0->M;

@@ -295,6 +295,7 @@ int build_context(aim_ctx* c, const aim_mesh* mesh) {
     Nc *= c->n[d];
     Lprod *= c->L[d];
   }
+  c->px = row_pitch(c->n[0], c->opts.mem_budget);
   // strided (y, z) passes: a four-step length up to 1296, any other 2,3,5-smooth length up to 900 (the
   // Stockham kernel's shared-memory limit)
   int l1 = 0, l2 = 0;
