@@ -317,10 +317,11 @@ template <class F> static void interp_shape(bool mf, int nrhs, bool warp, F&& f)
   else rhs(std::false_type{});
 }
 
-// out[c][r] = in[r][c] for an R x Cn row-major matrix (32 x 32 tiles through
-// shared memory, so both the reads and the writes are coalesced).
+// out[c][r] = in[r][c] for an R x Cn row-major matrix, rows of out ldo apart (32 x 32 tiles
+// through shared memory, so both the reads and the writes are coalesced).
 template <class E>
-__global__ void __launch_bounds__(256) k_transpose(const E* __restrict__ in, E* __restrict__ out, int R, long long Cn) {
+__global__ void __launch_bounds__(256) k_transpose(const E* __restrict__ in, E* __restrict__ out, int R, long long Cn,
+                                                   int ldo) {
   pdl_begin();
   __shared__ E t[32][33];
   const long long c0 = blockIdx.x * 32LL;
@@ -334,15 +335,53 @@ __global__ void __launch_bounds__(256) k_transpose(const E* __restrict__ in, E* 
   for (int i = threadIdx.y; i < 32; i += 8) {
     const long long cc = c0 + i;
     const int r = r0 + threadIdx.x;
-    if (r < R && cc < Cn) out[cc * R + r] = t[threadIdx.x][i];
+    if (r < R && cc < Cn) out[cc * ldo + r] = t[threadIdx.x][i];
   }
 }
 
 template <class E>
-static int transpose(aim_ctx* c, const char* name, const E* in, E* out, int R, long long Cn) {
+static int transpose(aim_ctx* c, const char* name, const E* in, E* out, int R, long long Cn, int ldo) {
   dim3 grid((unsigned)((Cn + 31) / 32), (unsigned)((R + 31) / 32));
-  AIM_LAUNCH(c, name, (launch_pdl(sizeof(E) <= 8, k_transpose<E>, grid, dim3(32, 8), 0, c->stream, in, out, R, Cn)));
+  AIM_LAUNCH(c, name,
+             (launch_pdl(sizeof(E) <= 8, k_transpose<E>, grid, dim3(32, 8), 0, c->stream, in, out, R, Cn, ldo)));
   return launch_check(c, name);
+}
+
+// How the many-RHS kernels lay B right-hand sides over lanes: LG lanes (a warp or half of one) per
+// node or row group, RL consecutive right-hand sides each, RHS-minor rows of ld of them.  Two a
+// lane need rows of an even length (16-byte loads), so an odd B takes one more column; without the
+// room for it (a memory budget, whose plan has max_rhs columns) a lane takes one.  Up to 16 RL
+// right-hand sides fit half a warp, which then serves two groups at a time: 33 right-hand sides
+// took a second pass of every warp for one lane (30.5 lambda plate: interpolation 808 us), 17 left
+// half of the lanes idle.
+// A body with few row groups (under eight for every SM) keeps a warp to each: it waits for its chain
+// of gathers, which half as many warps only lengthen (176 unknowns, 31 right-hand sides: 22 us, 30).
+struct RhsLanes {
+  int rl, lg, ld;
+};
+static int rhs_columns(const aim_ctx* c) { return c->max_rhs + (c->max_rhs % 2 && c->opts.mem_budget == 0 ? 1 : 0); }
+static RhsLanes rhs_lanes(const aim_ctx* c, int B) {
+  const int even = B + B % 2;
+  const bool few = c->N < 152 * 8 * kNearGroup && B <= 32;
+  RhsLanes r{};
+  r.rl = B > 16 && !few && even <= rhs_columns(c) ? 2 : 1;
+  r.lg = B <= 16 * r.rl && !few ? 16 : 32;
+  r.ld = r.rl == 2 ? even : B;
+  return r;
+}
+// Calls f(RL, LG) with the layout's numbers as types.
+template <class F> static void with_lanes(const RhsLanes& r, F&& f) {
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  using H = std::integral_constant<int, 16>;
+  using W = std::integral_constant<int, 32>;
+  if (r.rl == 2) {
+    if (r.lg == 16) f(I2{}, H{});
+    else f(I2{}, W{});
+  } else {
+    if (r.lg == 16) f(I1{}, H{});
+    else f(I1{}, W{});
+  }
 }
 
 // RL consecutive complex values as one load (16 bytes for two complex64).
@@ -415,17 +454,21 @@ __device__ __forceinline__ GroupVals<double2> load_group(const double2* p) {
 static_assert(kNearGroup == 4, "load_group reads four entries");
 
 // Interpolation + near correction for many right-hand sides over groups of
-// kNearGroup consecutive basis functions: one warp per group, lanes over
-// right-hand sides (RL consecutive ones per lane) on RHS-minor Phi and x.
+// kNearGroup consecutive basis functions: LG lanes per group, over
+// right-hand sides (RL consecutive ones per lane) on RHS-minor Phi and x
+// with rows of ld.
 // The grid part runs row by row (each stencil node's four grid values are
 // contiguous runs of right-hand sides; weights warp-uniform); the near part walks
 // the group's union of columns, so each x run is gathered once per group
 // rather than once per row that holds the column (neighbouring basis
 // functions share most of their near zone), at the price of multiplying the
-// zeros of the rows that lack a column.  The block's 32 rows of y are staged
-// in shared memory and written back in the [B][N] layout.
-template <class MI, int RL, bool MF>
-__global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R>* __restrict__ PhiT,
+// zeros of the rows that lack a column.  The block's rows of y are staged
+// in shared memory and written back in the [B][N] layout.  Bound by the latency
+// of the runs' gathers, so complex64 keeps to 64 registers (80 with the MFIE
+// weights) for the warps' sake, with some values spilled (32 lambda plate, 64
+// right-hand sides: 911 us at 88 registers, 695 at 64).
+template <class MI, int RL, bool MF, int LG>
+__global__ void __launch_bounds__(256, sizeof(typename MI::R) > 4 ? 1 : MF ? 3 : 4) interp_near_grp(const cplx<typename MI::R>* __restrict__ PhiT,
                                                        const cplx<typename MI::R>* __restrict__ xT,
                                                        cplx<typename MI::R>* __restrict__ y,
                                                        const typename MI::R* __restrict__ lam,
@@ -433,20 +476,21 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
                                                        const int32_t* __restrict__ gptr,
                                                        const int32_t* __restrict__ gcol,
                                                        const cplx<typename MI::R>* __restrict__ gval, int N,
-                                                       long long Nc, int nx, int ny, int B, typename MI::R fvec,
-                                                       typename MI::R frho, int S, int P,
+                                                       long long Nc, int nx, int ny, int B, int ld,
+                                                       typename MI::R fvec, typename MI::R frho, int S, int P,
                                                        const typename MI::R* __restrict__ lamM, typename MI::R fmf) {
   pdl_begin();
   using R = typename MI::R;
   using C = cplx<R>;
   constexpr int G = kNearGroup;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* ys = reinterpret_cast<C*>(smem_raw);  // [8 G][B + 1] (a padded row: the write-back reads down a column)
+  constexpr int NG = 256 / LG;              // groups per block
+  C* ys = reinterpret_cast<C*>(smem_raw);  // [NG G][B + 1] (a padded row: the write-back reads down a column)
   const int YS = B + 1;
   __shared__ int s_off[kMaxStencil];
   stencil_offsets_smem(s_off, S, P, nx, ny);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long g = blockIdx.x * 8LL + warp;
+  const int grp = threadIdx.x / LG, lane = threadIdx.x & (LG - 1);
+  const long long g = blockIdx.x * (long long)NG + grp;
   const int m0 = (int)(g * G);
   if (m0 < N) {
     const int nr = min(G, N - m0);
@@ -455,9 +499,9 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
 #ifdef AIM_CHECK
     if (!indices_ok(gcol, u0, u1, N, 3)) u1 = u0;
 #endif
-    const long long cs = Nc * B;  // component stride of PhiT
-    for (int bc = 0; bc < B; bc += 32 * RL) {
-      const int b = bc + RL * lane;  // B is a multiple of RL
+    const long long cs = Nc * ld;  // component stride of PhiT
+    for (int bc = 0; bc < B; bc += LG * RL) {
+      const int b = bc + RL * lane;
       if (b >= B) continue;
       C acc[G][RL];
 #pragma unroll
@@ -482,7 +526,7 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
         for (int q = 0; q < RL; ++q) av[q] = ar[q] = am[q] = cmake<C>(0, 0);
 #pragma unroll 3
         for (int s = 0; s < Sc; ++s) {
-          const C* ph = PhiT + (b0 + (long long)s_off[s]) * B + b;
+          const C* ph = PhiT + (b0 + (long long)s_off[s]) * ld + b;
           const Run<C, RL> px = load_run<C, RL>(ph), py = load_run<C, RL>(ph + cs), pz = load_run<C, RL>(ph + 2 * cs),
                            pr = load_run<C, RL>(ph + 3 * cs);
           const R wx = lm[s], wy = lm[S + s], wz = lm[2 * S + s], wr = lm[3 * S + s];
@@ -522,7 +566,7 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
         for (int i = 0; i < EB; ++i) col[i] = gcol[u + i];
         Run<C, RL> xv[EB];
 #pragma unroll
-        for (int i = 0; i < EB; ++i) xv[i] = load_run<C, RL>(xT + (long long)col[i] * B + b);
+        for (int i = 0; i < EB; ++i) xv[i] = load_run<C, RL>(xT + (long long)col[i] * ld + b);
 #pragma unroll
         for (int i = 0; i < EB; ++i) {
           const GroupVals<C> gv = load_group(gval + (long long)(u + i) * G);
@@ -538,7 +582,7 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
         }
       }
       for (; u < u1; ++u) {
-        const Run<C, RL> xv = load_run<C, RL>(xT + (long long)gcol[u] * B + b);
+        const Run<C, RL> xv = load_run<C, RL>(xT + (long long)gcol[u] * ld + b);
         const GroupVals<C> gv = load_group(gval + (long long)u * G);
 #pragma unroll
         for (int r = 0; r < G; ++r) {
@@ -553,26 +597,27 @@ __global__ void __launch_bounds__(256) interp_near_grp(const cplx<typename MI::R
 #pragma unroll
       for (int r = 0; r < G; ++r)
 #pragma unroll
-        for (int q = 0; q < RL; ++q) ys[(warp * G + r) * YS + b + q] = acc[r][q];
+        for (int q = 0; q < RL; ++q)
+          if (b + q < B) ys[(grp * G + r) * YS + b + q] = acc[r][q];
     }
   }
   __syncthreads();
-  const long long mb = blockIdx.x * 8LL * G;
-  const int rows = (int)min(8LL * G, (long long)N - mb);
-  for (int t = threadIdx.x; t < 8 * G * B; t += blockDim.x) {
-    const int i = t % (8 * G), bb = t / (8 * G);
+  const long long mb = blockIdx.x * (long long)(NG * G);
+  const int rows = (int)min((long long)(NG * G), (long long)N - mb);
+  for (int t = threadIdx.x; t < NG * G * B; t += blockDim.x) {
+    const int i = t % (NG * G), bb = t / (NG * G);
     if (i < rows) y[(long long)bb * N + mb + i] = ys[i * YS + bb];
   }
 }
 
-// Projection for many right-hand sides: one warp per grid node, lanes over
+// Projection for many right-hand sides: LG lanes per grid node, over
 // right-hand sides (RL consecutive ones per lane) on the RHS-minor x, so each
 // entry's x values are one contiguous run; the entry's four weights are
 // warp-uniform.  A block's 32 nodes are staged in shared memory (node-major,
 // rows padded by one element against bank conflicts) and written back in the
 // [B][4][Nc] layout, 32 consecutive nodes per (RHS, component) row.  One
 // launch covers B right-hand sides of an x with ldx of them per row.
-template <class MD, int RL>
+template <class MD, int RL, int LG>
 __global__ void __launch_bounds__(256) proj_gather_rhs(const cplx<typename MD::R>* __restrict__ xT,
                                                        typename MD::S* __restrict__ Q, const int32_t* __restrict__ ptr,
                                                        const int32_t* __restrict__ mm,
@@ -584,9 +629,9 @@ __global__ void __launch_bounds__(256) proj_gather_rhs(const cplx<typename MD::R
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* qs = reinterpret_cast<C*>(smem_raw);  // [32][4 B + 1]
   const int NS = 4 * B + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = threadIdx.x / LG, lane = threadIdx.x & (LG - 1);
   const long long u0 = blockIdx.x * 32LL;
-  for (int i = warp; i < 32; i += 8) {
+  for (int i = grp; i < 32; i += 256 / LG) {
     const long long u = u0 + i;
     if (u >= Nc) break;
     const int e0 = ptr[u];
@@ -594,8 +639,8 @@ __global__ void __launch_bounds__(256) proj_gather_rhs(const cplx<typename MD::R
 #ifdef AIM_CHECK
     if (!indices_ok(mm, e0, e1, N, 1)) e1 = e0;
 #endif
-    for (int bc = 0; bc < B; bc += 32 * RL) {
-      const int b = bc + RL * lane;  // B is a multiple of RL
+    for (int bc = 0; bc < B; bc += LG * RL) {
+      const int b = bc + RL * lane;
       if (b >= B) continue;
       C a[4][RL];
 #pragma unroll
@@ -628,7 +673,8 @@ __global__ void __launch_bounds__(256) proj_gather_rhs(const cplx<typename MD::R
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc)
 #pragma unroll
-        for (int q = 0; q < RL; ++q) qs[i * NS + cc * B + b + q] = a[cc][q];
+        for (int q = 0; q < RL; ++q)
+          if (b + q < B) qs[i * NS + cc * B + b + q] = a[cc][q];
     }
   }
   __syncthreads();
@@ -923,6 +969,14 @@ static int ensure_near_groups(aim_ctx* c, PrecData<R>& pd) {
   return AIM_OK;
 }
 
+// RHS-minor copies of Phi and x for the many-RHS kernels (rhs_columns per row).
+template <typename R> static int ensure_rhs_minor(aim_ctx* c, PrecData<R>& pd) {
+  const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2], cols = rhs_columns(c);
+  if (!pd.phiT) AIM_CUDA_TRY(cudaMalloc(&pd.phiT, sizeof(cplx<R>) * cols * 4 * Nc));
+  if (!pd.xT) AIM_CUDA_TRY(cudaMalloc(&pd.xT, sizeof(cplx<R>) * cols * c->N));
+  return AIM_OK;
+}
+
 // MD: storage of the projected grid; MI: storage of Phi read by the interpolation.
 template <class MD, class MI>
 static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename MD::R>* y, int nrhs,
@@ -931,37 +985,32 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
   using R = typename MD::R;
   const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2];
   const bool many = nrhs >= kRhsLanesMin;
-  // two right-hand sides per lane once a warp has 64 to cover
-  const bool two = nrhs >= 64 && nrhs % 2 == 0;
+  const RhsLanes rl = rhs_lanes(c, nrhs);
   PrecData<R>& pd = prec_data<R>(c);
   if (many) {
-    if (!pd.phiT) {
-      AIM_CUDA_TRY(cudaMalloc(&pd.phiT, sizeof(cplx<R>) * c->max_rhs * 4 * Nc));
-      AIM_CUDA_TRY(cudaMalloc(&pd.xT, sizeof(cplx<R>) * c->max_rhs * c->N));
-    }
-    AIM_TRY(transpose(c, "transpose_x", x, pd.xT, nrhs, (long long)c->N));
+    AIM_TRY(ensure_rhs_minor(c, pd));
+    AIM_TRY(transpose(c, "transpose_x", x, pd.xT, nrhs, (long long)c->N, rl.ld));
     // right-hand sides per launch: up to 64, shared memory 32 (4 B + 1) elements
     const int chunk = std::min(nrhs, 64);
     const size_t sm = sizeof(cplx<R>) * 32 * (4 * chunk + 1);
     const int blocks = (int)((Nc + 31) / 32);
-    static const cudaError_t attr1 = cudaFuncSetAttribute(proj_gather_rhs<MD, 1>,
-                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    static const cudaError_t attr2 = cudaFuncSetAttribute(proj_gather_rhs<MD, 2>,
-                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    AIM_CUDA_TRY(attr1);
-    AIM_CUDA_TRY(attr2);
     for (int b0 = 0; b0 < nrhs; b0 += chunk) {
       const int nb = std::min(chunk, nrhs - b0);
       const cplx<R>* xs = pd.xT + b0;
       typename MD::S* qd = grid0 + (long long)b0 * 4 * Nc;
-      if (nb == 64 && nrhs % 2 == 0)  // two per lane: 16-byte loads need an even row stride
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather_rhs<MD, 2>, blocks, 256, sm, c->stream, xs, qd, c->pnode_ptr,
-                                                                                            c->pnode_m, pw, Nc, nb,
-                                                                                            nrhs, c->N)));
-      else
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather_rhs<MD, 1>, blocks, 256, sm, c->stream, xs, qd, c->pnode_ptr,
-                                                                                            c->pnode_m, pw, Nc, nb,
-                                                                                            nrhs, c->N)));
+      int rc = AIM_OK;
+      with_lanes(RhsLanes{rl.rl, nrhs <= 64 || nb > 16 * rl.rl ? rl.lg : 16, rl.ld}, [&](auto l, auto w) {
+        const auto kern = proj_gather_rhs<MD, decltype(l)::value, decltype(w)::value>;
+        static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (attr != cudaSuccess) {
+          set_error(std::string("proj_gather: ") + cudaGetErrorString(attr));
+          rc = AIM_ECUDA;
+          return;
+        }
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, kern, blocks, 256, sm, c->stream, xs, qd,
+                                                 c->pnode_ptr, c->pnode_m, pw, Nc, nb, rl.ld, c->N)));
+      });
+      AIM_TRY(rc);
       AIM_TRY(launch_check(c, "proj_gather"));
     }
   } else {
@@ -983,31 +1032,33 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
   }
   AIM_TRY(convolve(c, 4 * nrhs));
   if (many) {
-    AIM_TRY(transpose(c, "transpose_phi", reinterpret_cast<const cplx<R>*>(phi), pd.phiT, nrhs, 4 * Nc));
+    AIM_TRY(transpose(c, "transpose_phi", reinterpret_cast<const cplx<R>*>(phi), pd.phiT, nrhs, 4 * Nc, rl.ld));
     AIM_TRY(ensure_near_groups(c, pd));
-    const int blocks = (int)((c->N + 8 * kNearGroup - 1) / (8 * kNearGroup));
-    const size_t sm = sizeof(cplx<R>) * 8 * kNearGroup * (nrhs + 1);
     const R fvec = (R)(c->alpha * c->k * kEta0), frho = (R)(c->alpha * kEta0 / c->k),
             fmf = (R)((1.0 - c->alpha) * kEta0);
-    const auto go = [&](auto mf, auto rl) {
-      constexpr bool MF = decltype(mf)::value;
-      constexpr int RL = decltype(rl)::value;
-      // staged rows: at most 32 x 256 complex128 (128 KB), beside the stencil offsets
-      static const cudaError_t attr = cudaFuncSetAttribute(interp_near_grp<MI, RL, MF>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      AIM_CUDA_TRY(attr);
-      AIM_LAUNCH(c, "interp_near",
-                 (launch_pdl(sizeof(typename MI::R) == 4, interp_near_grp<MI, RL, MF>, blocks, 256, sm, c->stream, 
-                     pd.phiT, pd.xT, y, lam, c->base, c->ngrp_ptr, c->ngrp_col, pd.ngrp_val, c->N, Nc, c->n[0],
-                     c->n[1], nrhs, fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
-      return AIM_OK;
+    int rc = AIM_OK;
+    const auto go = [&](auto mf) {
+      with_lanes(rl, [&](auto l, auto w) {
+        constexpr bool MF = decltype(mf)::value;
+        constexpr int RL = decltype(l)::value, LG = decltype(w)::value, rows = 256 / LG * kNearGroup;
+        const auto kern = interp_near_grp<MI, RL, MF, LG>;
+        const int blocks = (c->N + rows - 1) / rows;
+        const size_t sm = sizeof(cplx<R>) * rows * (nrhs + 1);
+        // staged rows: at most 32 x 256 complex128 (128 KB), beside the stencil offsets
+        static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (attr != cudaSuccess) {
+          set_error(std::string("interp_near: ") + cudaGetErrorString(attr));
+          rc = AIM_ECUDA;
+          return;
+        }
+        AIM_LAUNCH(c, "interp_near",
+                   (launch_pdl(sizeof(typename MI::R) == 4, kern, blocks, 256, sm, c->stream, pd.phiT, pd.xT, y, lam,
+                               c->base, c->ngrp_ptr, c->ngrp_col, pd.ngrp_val, c->N, Nc, c->n[0], c->n[1], nrhs, rl.ld,
+                               fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
+      });
     };
-    using T2 = std::integral_constant<int, 2>;
-    using T1 = std::integral_constant<int, 1>;
-    if (pd.lamM)
-      AIM_TRY(two ? go(std::true_type{}, T2{}) : go(std::true_type{}, T1{}));
-    else
-      AIM_TRY(two ? go(std::false_type{}, T2{}) : go(std::false_type{}, T1{}));
+    if (pd.lamM) go(std::true_type{}); else go(std::false_type{});
+    AIM_TRY(rc);
     return launch_check(c, "interp_near");
   }
   {
@@ -1066,15 +1117,8 @@ int prepare_product(aim_ctx* c, int precision) {
   AIM_TRY(ensure_grids(c, precision));
   if (precision == AIM_C128) return ensure_ff_arrays(c);
   if (c->max_rhs >= kRhsLanesMin) {
-    const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2];
-    if (precision == AIM_C64 && !c->p32.phiT) {
-      AIM_CUDA_TRY(cudaMalloc(&c->p32.phiT, sizeof(float2) * c->max_rhs * 4 * Nc));
-      AIM_CUDA_TRY(cudaMalloc(&c->p32.xT, sizeof(float2) * c->max_rhs * c->N));
-    }
-    if (precision == AIM_C128_F64 && !c->p64.phiT) {
-      AIM_CUDA_TRY(cudaMalloc(&c->p64.phiT, sizeof(double2) * c->max_rhs * 4 * Nc));
-      AIM_CUDA_TRY(cudaMalloc(&c->p64.xT, sizeof(double2) * c->max_rhs * c->N));
-    }
+    if (precision == AIM_C64) AIM_TRY(ensure_rhs_minor(c, c->p32));
+    if (precision == AIM_C128_F64) AIM_TRY(ensure_rhs_minor(c, c->p64));
     if (precision == AIM_C64) AIM_TRY(ensure_near_groups(c, c->p32));
     if (precision == AIM_C128_F64) AIM_TRY(ensure_near_groups(c, c->p64));
   }
