@@ -254,7 +254,10 @@ int aim_mie_sigma_thth(double radius, double k, int ndir, const double* theta, c
  * AIM_C64 counts the complex64 grids and the float-float grids of the
  * FP64-accurate refinement, AIM_C128 the float-float grids, AIM_C128_F64 the
  * native FP64 grids; cfie_alpha as in aim_opts (1: EFIE; < 1 adds the MFIE
- * arrays).  Not included: the fixed 64 MiB array of aim_matvec_c64_noalloc.
+ * arrays).  Not included: the fixed 64 MiB array of aim_matvec_c64_noalloc,
+ * and, for a context without a mem_budget, the padding of the transformed
+ * grids' rows and of the many-RHS vectors (under 5 %) and the workspace that
+ * aim_rcs keeps between calls (at most 64 MiB).
  * Host only.  AIM_EINVAL for a bad argument or a mesh with non-finite vertex
  * coordinates. */
 int aim_footprint(const aim_mesh* mesh, double h, int M, double near_radius, int max_rhs, double cfie_alpha,

@@ -303,16 +303,17 @@ struct LaunchScope {
     ::aim::LaunchScope _ls((ctx), (name)); \
     __VA_ARGS__;                          \
   } while (0)
-// Kernels of a product (and of an Arnoldi step) are launched so that one may be
-// set up while the previous one still runs (programmatic stream
-// serialisation): each first allows its successor the same and then waits for
-// its predecessor to be complete and its writes visible, before it touches
-// memory.  A kernel that is not launched this way starts and ends as usual.
-// A 1 lambda plate's six launches: 32.8 -> 22.4 us.  Not for kernels bound by the
-// FP64 pipe (overlap = false, and the solver's): blocks that start while others
-// still run land unevenly on the SMs, and each SM has its own two FP64 lanes a
-// clock (a 4 lambda plate in native FP64: 77 -> 146 us).  Nor for a launch larger than one
-// wave, which gains nothing (32 lambda plate, 64 right-hand sides: 1.70 -> 1.73 ms).
+// The kernels of a small product are launched so that one may be set up while
+// the previous one still runs (programmatic stream serialisation): each first
+// allows its successor the same and then waits for its predecessor to be
+// complete and its writes visible, before it touches memory.  A kernel that is
+// not launched this way starts and ends as usual.  A 1 lambda plate's six
+// launches: 32.8 -> 22.4 us.  Not for kernels bound by the FP64 pipe (overlap =
+// false; the solver's launches are plain): blocks that start while others still
+// run land unevenly on the SMs, each of which has its own two FP64 lanes a
+// clock (a 4 lambda plate in native FP64: 77 -> 146 us).  Nor for a launch
+// larger than one wave, which gains nothing (32 lambda plate, 64 right-hand
+// sides: 1.70 -> 1.73 ms).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -8,8 +8,9 @@
 // (X[k1 + L1 k2] = sum_n2 w_L2^(n2 k2) w_L^(n2 k1) sum_n1 x[L2 n1 + n2] w_L1^(n1 k1).)
 // Compared with one shared-memory round trip per radix stage, a pencil makes
 // one round trip (two for the fused forward-product-inverse x pass) and all
-// index arithmetic inside the register DFTs is resolved at compile time.  These kernels serve the padded lengths in
-// kFourStepLengths; other lengths use the Stockham kernels of fft.cu.
+// index arithmetic inside the register DFTs is resolved at compile time.
+// These kernels serve the padded lengths of AIM_FOURSTEP_LENGTHS; longer ones
+// use the Stockham kernels of fft.cu.
 //
 // Twiddles: twL holds w_L^t for t < L (the Stockham kernels' table), then
 // the same factors w_L^(k1 n2) laid out twice for the four-step kernels: as
@@ -191,13 +192,14 @@ __global__ void __launch_bounds__(strided_threads<P, L1, L2>(), strided_min_bloc
 //   step C (unit n2, to global):     column n2: inverse DFT_L1, samples < nx written.
 // One [L1][odd L2] tile per pencil, two shared-memory round trips.  (Both
 // twiddle products in step B, from one table, lengthen the longest step: 648^3
-// 24.1 -> 30.9 ms.  Two pencils a thread with all operations packed halves the
+// 24.8 -> 30.9 ms.  Two pencils a thread with all operations packed halves the
 // instructions and leaves too few warps: 27.7 ms.)  The block handles RY rows (ky)
 // x TG grids at a time, in as many rounds of its threads as each step's units
 // take (one where the split is even), and keeps the RY rows of Ghat in shared
 // memory.  Complex64 is bound by the L1/shared-memory pipe and the latency of
 // the rounds, so it runs in small blocks, whose barriers hold up fewer warps
-// (648^3, 32 grids: 24.1 ms in 128-thread blocks, 26.5 in 256); the 16-byte
+// (648^3, 32 grids: 24.8 ms in 128-thread blocks, 26.5 in 256; 64 and 96 threads:
+// 5 and 14 % slower); the 16-byte
 // policies are bound by the FP32 or FP64 pipe.
 template <class P> constexpr int x_threads() { return sizeof(typename P::S) <= 8 ? 128 : 256; }
 // Resident blocks per SM the register allocation must allow.

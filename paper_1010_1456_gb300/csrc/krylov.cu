@@ -354,8 +354,8 @@ int alloc_krylov(aim_ctx* c) {
   // norm kernel: about four blocks per SM over all right-hand sides, at least 256 elements per block
   k.nblk = std::max(1, std::min((4 * 152 + B - 1) / B, (N + 255) / 256));
   // dot kernel: at least 512 elements per block, about two blocks per SM per vector group (its
-  // FP64 work has to reach every SM: with 1024 the second vector group of two right-hand sides of
-  // 14,520 unknowns was the first to fill the GPU)
+  // FP64 work has to reach every SM: 1024 gave a vector group of two right-hand sides of 14,520
+  // unknowns 30 blocks for 152 SMs)
   k.nblk_dot = std::max(1, std::min((2 * 152 + B - 1) / B, (N + 511) / 512));
   k.nblk_upd = std::min(1024, (N + kUpdThreads - 1) / kUpdThreads);
   const int nb = std::max(std::max(k.nblk, k.nblk_dot), k.nblk_upd);

@@ -182,8 +182,10 @@ constexpr int kMaxStencil = 216;
 // latency of its gathers (stencil nodes of Phi, columns of x), so a chunk of
 // right-hand sides keeps BC times as many in flight and reads the weights, the
 // near entries and their columns once for all of them (16 lambda sphere, 8
-// right-hand sides: 1.82 -> 1.38 ms); a small body takes a whole warp per basis function, which leaves one or two rounds of gathers
-// where 8 lanes take five to ten.
+// right-hand sides: 1.82 -> 1.38 ms; 7 lambda sphere, CFIE, 4: 267 -> 206 us,
+// at 64 registers, for the warps' sake); a small body takes a whole warp per
+// basis function, which leaves one or two rounds of gathers where 8 lanes take
+// five to ten.
 template <class MD, bool MF, int BC, int W>
 __global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 ? 4 : 2) interp_near(const typename MD::S* __restrict__ Phi,
                                                    const cplx<typename MD::R>* __restrict__ x,
