@@ -93,10 +93,13 @@ struct ProjTasks {
 // start).  The next task's list bounds are loaded while the current one is
 // summed, and the right-hand sides go in chunks of BC: an entry's weights
 // and column are loaded once per chunk and its BC gathers of x are
-// independent loads.  U entries are in flight per lane: two where the tasks
-// are a single wave of blocks, which then only wait for their loads (a 5
-// lambda plate, 4 right-hand sides: 10.9 -> 9.0 us), one beyond, where the
+// independent loads.  U entries are in flight per lane, as many as leave the
+// registers for full residency (one right-hand side: 64 lambda plate, 51 us
+// with one entry, 45 with four; 10 lambda sphere, 97 us, 91).  Four right-hand
+// sides take two where the tasks are a single wave of blocks, which then only
+// wait for their loads (a 5 lambda plate: 10.9 -> 9.0 us), one beyond, where the
 // registers of a second cost resident warps (7 lambda sphere: 107 us, 127).
+constexpr int gather_unroll(int bc, bool one_wave) { return bc == 1 ? 4 : one_wave ? 2 : bc == 2 ? 4 : 1; }
 template <class MD, int BC, int U>
 __global__ void __launch_bounds__(256) proj_gather(const cplx<typename MD::R>* __restrict__ x, typename MD::S* __restrict__ Q,
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ mm,
@@ -269,7 +272,9 @@ __global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 ? 4 : 2) inte
       }
     }
     const C* xb = x + (long long)bc * N;
-#pragma unroll 2
+    // entries in flight: four where a single complex64 right-hand side leaves the registers (64 lambda
+    // plate: 308 us with two, 274 with four), two otherwise
+#pragma unroll(sizeof(R) == 4 && BC == 1 ? 4 : 2)
     for (int e = r0 + lane; e < r1; e += W) {
       const C v = nval[e];
       const C* xc = xb + ncol[e];
@@ -1020,11 +1025,12 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const int32_t* groups = c->sparse_proj ? c->pgroups : nullptr;
     const auto go = [&](auto bc) {
+      constexpr int BC = decltype(bc)::value;
       if (blocks <= 2 * 152)
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, decltype(bc)::value, 2>, blocks, 256, 0, c->stream, 
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll(BC, true)>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
       else
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, decltype(bc)::value, 1>, blocks, 256, 0, c->stream, 
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll(BC, false)>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
     };
     if (nrhs == 1) go(std::integral_constant<int, 1>{});
@@ -1182,7 +1188,8 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
     const long long ntask = (Nc + 7) / 8;
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const auto go = [&](auto bc) {
-      AIM_LAUNCH(c, "proj_gather", (launch_pdl(true, proj_gather<M32, decltype(bc)::value, 1>, blocks, 256, 0, c->stream, 
+      constexpr int BC = decltype(bc)::value;
+      AIM_LAUNCH(c, "proj_gather", (launch_pdl(true, proj_gather<M32, BC, gather_unroll(BC, false)>, blocks, 256, 0, c->stream, 
                                        x, g0, c->pnode_ptr, c->pnode_m, c->p32.pnode_w, c->N, Nc, nrhs, nullptr,
                                        ntask)));
     };
