@@ -321,7 +321,11 @@ int aim_probe_fma_peak(int which, double* tflops);
  * five passes of the convolution (z forward, y forward, the fused x pass --
  * forward transform, spectral product, inverse -- y inverse, z inverse, in
  * that order) runs one of:
- *   AIM_FFT_AUTO            the built-in rule (default): four-step;
+ *   AIM_FFT_AUTO            the built-in rule (default): four-step where the padded
+ *                           length has such a kernel, except Stockham for x passes
+ *                           of AIM_C128 and AIM_C128_F64 with few pencils and
+ *                           register DFTs of 24 points or more (padded x lengths
+ *                           125, 243, 250, 375 and from 384 on all but 400);
  *   AIM_FFT_STOCKHAM        mixed-radix Stockham kernel (any 2,3,5-smooth length);
  *   AIM_FFT_FOURSTEP        four-step register kernel (every padded length up to
  *                           900 and 1296; a longer one falls back to the
@@ -332,7 +336,8 @@ int aim_probe_fma_peak(int which, double* tflops);
  *   AIM_FFT_FOURSTEP_WARP, AIM_FFT_FOURSTEP_WIDE  accepted; run as
  *                           AIM_FFT_FOURSTEP.
  * aim_fft_config sets (set != NULL, [5]) and/or reads (get != NULL, [5]) the
- * choices of one precision; get receives them with AUTO resolved by the rule.
+ * choices of one precision; get receives them with AUTO resolved by the rule
+ * for products of max_rhs vectors.
  */
 enum {
   AIM_FFT_AUTO = 0,

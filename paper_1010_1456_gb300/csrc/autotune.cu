@@ -74,11 +74,14 @@ static int autotune(aim_ctx* c, int precision, int nrhs, int reps, int32_t* kern
     for (int i = 0; i < AIM_FFT_PASSES * AIM_FFT_KERNELS; ++i) ms_out[i] = -1.0;
   for (int pass = 0; pass < AIM_FFT_PASSES && rc == AIM_OK; ++pass) {
     if ((pass == 0 || pass == 4) && c->L[2] == 1) continue;  // a planar grid has no z passes
-    int best = AIM_FFT_AUTO;
+    const int axis = pass == 2 ? 0 : pass == 1 || pass == 3 ? 1 : 2;
+    int l1 = 0, l2 = 0, best = AIM_FFT_AUTO;
+    const bool fourstep = fourstep_split(c->L[axis], &l1, &l2);  // else every choice runs Stockham
     double best_ms = 0.0;
     for (int k = AIM_FFT_STOCKHAM; k < AIM_FFT_KERNELS && rc == AIM_OK; ++k) {
       // the x pass has a small-block variant; the warp-group and wide choices run the plain four-step kernel
       if (k == AIM_FFT_FOURSTEP_WARP || k == AIM_FFT_FOURSTEP_WIDE || (k == AIM_FFT_FOURSTEP_SMALL && pass != 2)) continue;
+      if (k != AIM_FFT_STOCKHAM && !fourstep) continue;
       c->fft_kernel[pol][pass] = k;
       double ms = 0.0;
       rc = time_pass(c, pass, x, y, nrhs, precision, reps, &ms);
@@ -96,7 +99,7 @@ static int autotune(aim_ctx* c, int precision, int nrhs, int reps, int32_t* kern
     c->fft_kernel[pol][pass] = best;
   }
   if (rc == AIM_OK && kernel_out)
-    for (int pass = 0; pass < AIM_FFT_PASSES; ++pass) kernel_out[pass] = fft_kernel_for(c, pol, pass);
+    for (int pass = 0; pass < AIM_FFT_PASSES; ++pass) kernel_out[pass] = fft_kernel_for(c, pol, pass, 4 * nrhs);
   cudaStreamSynchronize(c->stream);
   cudaFree(x);
   cudaFree(y);
@@ -123,7 +126,7 @@ extern "C" int aim_fft_config(aim_ctx* ctx, int precision, const int32_t* set, i
     drop_step_graph(ctx);
   }
   if (get)
-    for (int i = 0; i < AIM_FFT_PASSES; ++i) get[i] = fft_kernel_for(ctx, pol, i);
+    for (int i = 0; i < AIM_FFT_PASSES; ++i) get[i] = fft_kernel_for(ctx, pol, i, 4 * ctx->max_rhs);
   return AIM_OK;
 }
 

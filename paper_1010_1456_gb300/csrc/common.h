@@ -365,9 +365,9 @@ int fft_convolve_ff(aim_ctx* c, int G);
 // complex64 product and convolution on caller-provided grids (noalloc.cu)
 int fft_convolve_c64_bufs(aim_ctx* c, int G, float2* g0, float2* g1, float2* g2);
 // FFT kernel tables: policy index of a precision (0 complex64, 1 native FP64,
-// 2 float-float) and the kernel a pass runs (AIM_FFT_AUTO resolved).
+// 2 float-float) and the kernel a pass over G grids runs (AIM_FFT_AUTO resolved).
 int fft_policy_of(int precision);
-int fft_kernel_for(const aim_ctx* c, int pol, int pass);
+int fft_kernel_for(const aim_ctx* c, int pol, int pass, int G);
 int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0, float2* g1, float2* g2);
 int build_ghat(aim_ctx* c);
 // krylov.cu

@@ -26,6 +26,7 @@
 //   float-float (float4 = re.hi, im.hi, re.lo, im.lo; about 48 bits, on the
 //   FP32 pipes; see ff.h).  Per-stage index arithmetic uses precomputed
 //   multiply-shift division, so no integer division runs in the kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <type_traits>
@@ -375,9 +376,21 @@ bool fourstep_split(int L, int* L1, int* L2) {
 
 int fft_policy_of(int precision) { return precision == AIM_C64 ? 0 : precision == AIM_C128_F64 ? 1 : 2; }
 
-int fft_kernel_for(const aim_ctx* c, int pol, int pass) {
+// AIM_FFT_AUTO is the four-step kernel where the padded length has one, but for a few float-float or
+// FP64 pencils with long register DFTs in the x pass: too few units to hide their serial chains, and the
+// Stockham kernel's radix-5 and smaller steps use more threads (375 x 375 plane, 4 float-float grids: 54 us
+// four-step, 33 Stockham; 432: 35 and 33; FP64 135 and 107).  From 58 k units on the four-step kernel is the
+// faster one (648 x 648, 8 grids, 140 k units: 122 us, 164), and with DFTs of at most 20 it always was (320
+// plane, FP64: 70 and 77).
+int fft_kernel_for(const aim_ctx* c, int pol, int pass, int G) {
   const int k = c->fft_kernel[pol][pass];
-  return k != AIM_FFT_AUTO ? k : AIM_FFT_FOURSTEP;
+  if (k != AIM_FFT_AUTO) return k;
+  const int axis = pass == 2 ? 0 : pass == 1 || pass == 3 ? 1 : 2;
+  if (c->L[axis] == 1) return AIM_FFT_FOURSTEP;  // a planar grid's z passes, which do not run
+  int l1 = 0, l2 = 0;
+  if (!fourstep_split(c->L[axis], &l1, &l2)) return AIM_FFT_STOCKHAM;
+  const long long units = (long long)G * c->L[1] * c->L[2] * std::max(l1, l2);
+  return pass == 2 && pol != 0 && std::max(l1, l2) >= 24 && units < 384LL * 152 ? AIM_FFT_STOCKHAM : AIM_FFT_FOURSTEP;
 }
 
 template <class P> constexpr int policy_index() {
@@ -388,7 +401,7 @@ template <class P> constexpr int policy_index() {
 template <class P, bool INV, class O = typename P::S>
 static int strided_pass(aim_ctx* c, int pass, const char* name, const typename P::S* in, O* out,
                         const StridedArgs& a, int G, const FftPlan* plan_dev, int L, const typename P::S* tw) {
-  const int k = fft_kernel_for(c, policy_index<P>(), pass);
+  const int k = fft_kernel_for(c, policy_index<P>(), pass, G);
   if (k != AIM_FFT_STOCKHAM) {
     const int rc = Fft4<P>::strided(L, c, name, INV, in, out, a, G, L, tw);
     if (rc == 1) return AIM_OK;
@@ -400,7 +413,7 @@ static int strided_pass(aim_ctx* c, int pass, const char* name, const typename P
 template <class P>
 static int x_pass(aim_ctx* c, const char* name, typename P::S* buf, XArgs a, const FftPlan* plan_dev, int L,
                   const typename P::S* ghat, const typename P::S* tw) {
-  const int k = fft_kernel_for(c, policy_index<P>(), 2);
+  const int k = fft_kernel_for(c, policy_index<P>(), 2, a.G);
   if (k != AIM_FFT_STOCKHAM) {
     XArgs4 x4{};
     x4.nx = a.nx; x4.px = a.px; x4.Ly = a.rows_y; x4.Lz = a.rows_z; x4.G = a.G; x4.sG = a.sG; x4.hx = a.hx; x4.hy = a.hy;

@@ -66,12 +66,6 @@ int launch_x4(aim_ctx* c, const char* name, S* buf, XArgs4 a, const S* ghat, con
   constexpr int L = L1 * L2;
   constexpr long long per_pencil = pencil_stride(L1, L2, 128 / (int)sizeof(S));
   constexpr int LM = std::max(L1, L2);
-  // A few float-float or FP64 pencils with long register DFTs: too few units to hide their serial
-  // chains, and the Stockham kernel's radix-5 and smaller steps use more threads (375 x 375 plane,
-  // 4 float-float grids: 54 us here, 33 there; 432: 35 and 33; FP64 135 and 107).  From 58 k units
-  // on this kernel is the faster one (648 x 648, 8 grids, 140 k units: 122 us here, 164 there), and
-  // with DFTs of at most 20 it always was (320 plane, FP64: 70 and 77).
-  if (sizeof(S) > 8 && LM >= 24 && (long long)a.G * a.Ly * a.Lz * LM < 384LL * kSMs) return kNotHandled;
   const int T = std::min(threads, x_threads<Pol>());
   // shared memory of a block: an even share of an SM's among the resident blocks
   const long long cap = 220 * 1024 / (long long)sizeof(S) / (x_min_blocks<Pol, L1, L2>() * (x_threads<Pol>() / T));
