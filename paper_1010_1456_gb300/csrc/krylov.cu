@@ -358,7 +358,8 @@ int alloc_krylov(aim_ctx* c) {
   // unknowns 30 blocks for 152 SMs)
   k.nblk_dot = std::max(1, std::min((2 * 152 + B - 1) / B, (N + 511) / 512));
   k.nblk_upd = std::min(1024, (N + kUpdThreads - 1) / kUpdThreads);
-  const int nb = std::max(std::max(k.nblk, k.nblk_dot), k.nblk_upd);
+  // partial sums: the dot kernel's (GMRES) or the norm kernel's blocks (TFQMR); norms also the update kernel's
+  const int nb = std::max(k.nblk, k.nblk_dot), nb_norm = std::max(k.nblk, k.nblk_upd);
   const size_t vec = (size_t)N * sizeof(double2);
   AIM_CUDA_TRY(cudaMalloc(&k.V, vec * B * slots));
   k.slots = slots;
@@ -367,7 +368,7 @@ int alloc_krylov(aim_ctx* c) {
   AIM_CUDA_TRY(cudaMalloc(&k.H, sizeof(double2) * B * (m + 1) * m));
   AIM_CUDA_TRY(cudaMalloc(&k.partial, sizeof(double2) * B * nb * (m + 1 + kDotGroup)));
   AIM_CUDA_TRY(cudaMalloc(&k.y, sizeof(double2) * B * std::max(m, kTfqmrScalars)));
-  AIM_CUDA_TRY(cudaMalloc(&k.nrm, sizeof(double) * B * (2 + nb)));
+  AIM_CUDA_TRY(cudaMalloc(&k.nrm, sizeof(double) * B * (2 + nb_norm)));
   AIM_CUDA_TRY(cudaMalloc(&k.bnorm, sizeof(double) * B));
   AIM_CUDA_TRY(cudaMalloc(&k.active, sizeof(int) * B));
   AIM_CUDA_TRY(cudaMalloc(&k.reorth, sizeof(int) * B));
