@@ -77,6 +77,13 @@ __device__ __forceinline__ bool stencil_ok(long long base, int nx, int ny, long 
 }
 #endif
 
+// Frees what a failed set-up of several arrays got and clears the pointers, so the next call starts
+// over instead of running kernels on the arrays that are missing; also clears the runtime's last error.
+template <class... T> inline void release(T*&... p) {
+  ((cudaFree(p), p = nullptr), ...);
+  cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- complex
 template <typename R> struct cplx_t;
 template <> struct cplx_t<float> { using type = float2; };

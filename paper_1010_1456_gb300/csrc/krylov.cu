@@ -337,7 +337,7 @@ __global__ void k_xupdate(const double2* __restrict__ V, const double2* __restri
 }
 
 // ------------------------------------------------------------------ host driver
-int alloc_krylov(aim_ctx* c) {
+static int fill_krylov(aim_ctx* c) {
   KrylovWork& k = c->kw;
   const int B = c->max_rhs, m = c->opts.restart, N = c->N;
   // vectors per right-hand side: the GMRES basis, or the TFQMR vectors
@@ -397,6 +397,16 @@ void free_krylov(aim_ctx* c) {
   cudaFree(k.active); cudaFree(k.reorth); cudaFree(k.jdev); cudaFree(k.hcur); cudaFree(k.cnt);
   if (k.h_H) cudaFreeHost(k.h_H);
   k = KrylovWork{};
+}
+
+// All of the solver's storage or none of it.
+int alloc_krylov(aim_ctx* c) {
+  const int rc = fill_krylov(c);
+  if (rc != AIM_OK) {
+    free_krylov(c);
+    cudaGetLastError();
+  }
+  return rc;
 }
 
 namespace {

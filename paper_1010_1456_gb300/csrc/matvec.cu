@@ -873,9 +873,8 @@ __global__ void __launch_bounds__(256) interp_near_ff(const float4* __restrict__
 // Warp tasks of the projection: the listed groups, or every 8-node group.
 static long long proj_tasks(const aim_ctx* c, long long Nc) { return c->sparse_proj ? c->ngroups : (Nc + 7) / 8; }
 
-static int ensure_ff_arrays(aim_ctx* c) {
+static int fill_ff_arrays(aim_ctx* c) {
   FFData& p = c->pff;
-  if (p.pnode_w) return AIM_OK;
   const long long nent = c->nent, nl = (long long)c->N * 4 * c->S;
   AIM_CUDA_TRY(cudaMalloc(&p.pnode_w, sizeof(float4) * 2 * nent));
   AIM_CUDA_TRY(cudaMalloc(&p.lam, sizeof(float2) * nl));
@@ -897,6 +896,14 @@ static int ensure_ff_arrays(aim_ctx* c) {
     AIM_TRY(launch_check(c, "weights_to_ff"));
   }
   return AIM_OK;
+}
+
+static int ensure_ff_arrays(aim_ctx* c) {
+  FFData& p = c->pff;
+  if (p.pnode_w) return AIM_OK;
+  const int rc = fill_ff_arrays(c);
+  if (rc != AIM_OK) release(p.pnode_w, p.lam, p.near_val, p.xff, p.lamM);
+  return rc;
 }
 
 static int run_product_ff(aim_ctx* c, const double2* x, double2* y, int nrhs) {
@@ -950,7 +957,7 @@ template <> PrecData<double>& prec_data<double>(aim_ctx* c) { return c->p64; }
 // The row groups of the many-RHS near product: the union columns once, the
 // entries of a precision on its first use.
 template <typename R>
-static int ensure_near_groups(aim_ctx* c, PrecData<R>& pd) {
+static int fill_near_groups(aim_ctx* c, PrecData<R>& pd) {
   const long long ng = ((long long)c->N + kNearGroup - 1) / kNearGroup;
   const unsigned blocks = (unsigned)((ng + 255) / 256);
   if (!c->ngrp_ptr) {
@@ -976,12 +983,29 @@ static int ensure_near_groups(aim_ctx* c, PrecData<R>& pd) {
   return AIM_OK;
 }
 
+template <typename R>
+static int ensure_near_groups(aim_ctx* c, PrecData<R>& pd) {
+  if (c->ngrp_ptr && pd.ngrp_val) return AIM_OK;
+  const bool had = c->ngrp_ptr != nullptr;
+  const int rc = fill_near_groups(c, pd);
+  if (rc != AIM_OK) {
+    release(pd.ngrp_val);
+    if (!had) release(c->ngrp_ptr, c->ngrp_col);
+  }
+  return rc;
+}
+
 // RHS-minor copies of Phi and x for the many-RHS kernels (rhs_columns per row).
 template <typename R> static int ensure_rhs_minor(aim_ctx* c, PrecData<R>& pd) {
   const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2], cols = rhs_columns(c);
-  if (!pd.phiT) AIM_CUDA_TRY(cudaMalloc(&pd.phiT, sizeof(cplx<R>) * cols * 4 * Nc));
-  if (!pd.xT) AIM_CUDA_TRY(cudaMalloc(&pd.xT, sizeof(cplx<R>) * cols * c->N));
-  return AIM_OK;
+  if (pd.xT) return AIM_OK;
+  const int rc = [&]() -> int {
+    AIM_CUDA_TRY(cudaMalloc(&pd.phiT, sizeof(cplx<R>) * cols * 4 * Nc));
+    AIM_CUDA_TRY(cudaMalloc(&pd.xT, sizeof(cplx<R>) * cols * c->N));
+    return AIM_OK;
+  }();
+  if (rc != AIM_OK) release(pd.phiT, pd.xT);
+  return rc;
 }
 
 // MD: storage of the projected grid; MI: storage of Phi read by the interpolation.
@@ -1089,35 +1113,27 @@ int ensure_grids(aim_ctx* c, int precision) {
   const long long B = c->max_rhs;
   const long long nx = c->n[0], ny = c->n[1], nz = c->n[2], Ly = c->L[1], Lz = c->L[2], px = c->px;
   const long long e0 = B * 4 * nz * ny * nx, e1 = B * 4 * Lz * ny * px, e2 = B * 4 * Lz * Ly * px;
-  if (precision == AIM_C64) {
-    PrecData<float>& p = c->p32;
-    if (!p.grid0) {
-      AIM_TRY(budget_grids(c, precision));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid0, sizeof(float2) * e0));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid1, sizeof(float2) * e1));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid2, sizeof(float2) * e2));
-      if (c->sparse_proj) AIM_CUDA_TRY(cudaMemsetAsync(p.grid0, 0, sizeof(float2) * e0, c->stream));
+  const auto get = [&](auto& p) -> int {  // all three grids or none
+    if (p.grid0) return AIM_OK;
+    using E = std::remove_reference_t<decltype(*p.grid0)>;
+    const size_t planned = c->planned_bytes;
+    AIM_TRY(budget_grids(c, precision));
+    const int rc = [&]() -> int {
+      AIM_CUDA_TRY(cudaMalloc(&p.grid0, sizeof(E) * e0));
+      AIM_CUDA_TRY(cudaMalloc(&p.grid1, sizeof(E) * e1));
+      AIM_CUDA_TRY(cudaMalloc(&p.grid2, sizeof(E) * e2));
+      if (c->sparse_proj) AIM_CUDA_TRY(cudaMemsetAsync(p.grid0, 0, sizeof(E) * e0, c->stream));
+      return AIM_OK;
+    }();
+    if (rc != AIM_OK) {
+      release(p.grid0, p.grid1, p.grid2);
+      c->planned_bytes = planned;
     }
-  } else if (precision == AIM_C128_F64) {
-    PrecData<double>& p = c->p64;
-    if (!p.grid0) {
-      AIM_TRY(budget_grids(c, precision));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid0, sizeof(double2) * e0));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid1, sizeof(double2) * e1));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid2, sizeof(double2) * e2));
-      if (c->sparse_proj) AIM_CUDA_TRY(cudaMemsetAsync(p.grid0, 0, sizeof(double2) * e0, c->stream));
-    }
-  } else {
-    FFData& p = c->pff;
-    if (!p.grid0) {
-      AIM_TRY(budget_grids(c, precision));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid0, sizeof(float4) * e0));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid1, sizeof(float4) * e1));
-      AIM_CUDA_TRY(cudaMalloc(&p.grid2, sizeof(float4) * e2));
-      if (c->sparse_proj) AIM_CUDA_TRY(cudaMemsetAsync(p.grid0, 0, sizeof(float4) * e0, c->stream));
-    }
-  }
-  return AIM_OK;
+    return rc;
+  };
+  if (precision == AIM_C64) return get(c->p32);
+  if (precision == AIM_C128_F64) return get(c->p64);
+  return get(c->pff);
 }
 
 int prepare_product(aim_ctx* c, int precision) {
