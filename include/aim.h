@@ -99,7 +99,8 @@ typedef struct {
   size_t mem_budget; /* 0 (default): no limit.  Otherwise the most device memory, in bytes, the
                       context may plan to hold: aim_setup returns AIM_ENOMEM, before it allocates
                       anything, when aim_footprint's estimate for this mesh, max_rhs, cfie_alpha
-                      and precision exceeds it; a later product in a precision whose grids that
+                      and precision (less the padding that a context with a budget does without)
+                      exceeds it; a later product in a precision whose grids that
                       estimate does not include (see aim_footprint) returns AIM_ENOMEM when its
                       grids would take the planned total above the budget. */
   int krylov;        /* AIM_GMRES (default): restarted GMRES(restart); AIM_TFQMR: transpose-free QMR
@@ -254,10 +255,11 @@ int aim_mie_sigma_thth(double radius, double k, int ndir, const double* theta, c
  * AIM_C64 counts the complex64 grids and the float-float grids of the
  * FP64-accurate refinement, AIM_C128 the float-float grids, AIM_C128_F64 the
  * native FP64 grids; cfie_alpha as in aim_opts (1: EFIE; < 1 adds the MFIE
- * arrays).  Not included: the fixed 64 MiB array of aim_matvec_c64_noalloc,
- * and, for a context without a mem_budget, the padding of the transformed
- * grids' rows and of the many-RHS vectors (under 5 %) and the workspace that
- * aim_rcs keeps between calls (at most 64 MiB).
+ * arrays).  The grids' rows and the many-RHS vectors are counted padded, as a
+ * context without a mem_budget holds them (one with a budget needs up to 6 %
+ * less of them).  Not included: the fixed 64 MiB array of
+ * aim_matvec_c64_noalloc, and the workspace that a context without a
+ * mem_budget keeps once it has computed a pattern (aim_rcs, at most 64 MiB).
  * Host only.  AIM_EINVAL for a bad argument or a mesh with non-finite vertex
  * coordinates. */
 int aim_footprint(const aim_mesh* mesh, double h, int M, double near_radius, int max_rhs, double cfie_alpha,

@@ -77,9 +77,10 @@ static bool mesh_finite(const aim_mesh* mesh) {
 }
 
 // Device bytes of a context for this mesh once it has solved in `precision`
-// (see aim_footprint in aim.h).
+// (see aim_footprint in aim.h); mem_budget as in its options (0: rows and
+// right-hand sides are padded).
 int footprint_estimate(const aim_mesh* mesh, double h, int M, double near_radius, int max_rhs, double alpha,
-                       int precision, size_t* bytes) {
+                       int precision, size_t mem_budget, size_t* bytes) {
   (void)near_radius;
   if (mesh->nv < 1 || mesh->nt < 1 || !mesh->verts || !mesh->tris) {
     set_error("aim_footprint: empty mesh");
@@ -111,7 +112,8 @@ int footprint_estimate(const aim_mesh* mesh, double h, int M, double near_radius
   const long long S = (long long)(M + 1) * (M + 1) * (M + 1);
   const long long nnz = N * 100LL;  // generous near-row length
   const long long nc = n[0] * n[1] * n[2];
-  const double cells = (double)max_rhs * 4 * (nc + L[2] * n[1] * n[0] + L[2] * L[1] * n[0]);
+  const long long px = n[0] < INT32_MAX ? row_pitch((int)n[0], mem_budget) : n[0];
+  const double cells = (double)max_rhs * 4 * (nc + L[2] * n[1] * px + L[2] * L[1] * px);
   double b = 0;
   b += (double)N * 4 * S * (8 + 4) * 2;                               // weights f64/f32 + node lists
   b += (double)nnz * (16 + 8 + 4);                                     // near values + columns
@@ -123,7 +125,7 @@ int footprint_estimate(const aim_mesh* mesh, double h, int M, double near_radius
   if (precision != AIM_C128_F64)
     b += (double)N * 4 * S * 8 * 2 + (double)nnz * 16;                 // float-float weights and near values
   if (max_rhs >= kRhsLanesMin) {
-    b += (double)max_rhs * (4.0 * nc + N) * 16;  // RHS-minor copies of Phi and x
+    b += (double)rhs_columns(max_rhs, mem_budget) * (4.0 * nc + N) * 16;  // RHS-minor copies of Phi and x
     // near row groups: union columns (about 0.4 nnz) with kNearGroup entries each, in the solver precision
     b += (double)N / kNearGroup * 4 + 0.4 * nnz * (4 + kNearGroup * (precision == AIM_C64 ? 8 : 16));
   }
@@ -234,7 +236,8 @@ int aim_setup(const aim_mesh* mesh, double k, double h, int M, double near_radiu
   }
   size_t planned = 0;
   if (o.mem_budget > 0) {
-    AIM_TRY(footprint_estimate(mesh, h, M, near_radius, o.max_rhs, o.cfie_alpha, o.precision, &planned));
+    AIM_TRY(footprint_estimate(mesh, h, M, near_radius, o.max_rhs, o.cfie_alpha, o.precision, o.mem_budget,
+                               &planned));
     if (planned > o.mem_budget) {
       set_error("aim_setup: footprint estimate " + std::to_string(planned) + " bytes exceeds mem_budget " +
                 std::to_string(o.mem_budget));
@@ -426,7 +429,7 @@ int aim_footprint(const aim_mesh* mesh, double h, int M, double near_radius, int
     set_error("aim_footprint: bad arguments");
     return AIM_EINVAL;
   }
-  return footprint_estimate(mesh, h, M, near_radius, max_rhs, cfie_alpha, precision, bytes);
+  return footprint_estimate(mesh, h, M, near_radius, max_rhs, cfie_alpha, precision, 0, bytes);
 }
 
 int aim_export(aim_ctx* c, int what, void* dst, size_t bytes) {

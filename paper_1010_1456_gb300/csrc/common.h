@@ -361,6 +361,9 @@ int convert_c64_to_c128(aim_ctx* c, const float2* in, double2* out, int64_t coun
 // 250 -> 190 us, y forward 422 -> 380); rows from 64 nodes, where the padding is under 5 %, and not
 // for a context with a memory budget, whose plan counts the rows as they are.
 inline int row_pitch(int nx, size_t mem_budget) { return nx >= 64 && mem_budget == 0 ? (nx + 3) / 4 * 4 : nx; }
+// Right-hand sides the RHS-minor copies of Phi and x have room for: an even number, so that two a
+// lane fit an odd batch (rhs_lanes), but for a context with a memory budget.
+inline int rhs_columns(int max_rhs, size_t mem_budget) { return max_rhs + (max_rhs % 2 && mem_budget == 0 ? 1 : 0); }
 // Phi's grid: grid2 for a context that projects over node groups, else grid0.
 template <class T> inline T* phi_grid(const aim_ctx* c, T* g0, T* g2) { return c->sparse_proj ? g2 : g0; }
 // The four-step split L = L1 * L2 of a padded length that has four-step
@@ -388,7 +391,7 @@ int alloc_krylov(aim_ctx* c);
 // api.cu: footprint estimate (aim_footprint), and the mem_budget check of the
 // grids of a product precision the setup's estimate did not count.
 int footprint_estimate(const aim_mesh* mesh, double h, int M, double near_radius, int max_rhs, double alpha,
-                       int precision, size_t* bytes);
+                       int precision, size_t mem_budget, size_t* bytes);
 size_t grid_bytes(const aim_ctx* c, int precision);
 int budget_grids(aim_ctx* c, int precision);
 // Allocates everything a product of this precision allocates lazily, so a

@@ -366,12 +366,11 @@ static int transpose(aim_ctx* c, const char* name, const E* in, E* out, int R, l
 struct RhsLanes {
   int rl, lg, ld;
 };
-static int rhs_columns(const aim_ctx* c) { return c->max_rhs + (c->max_rhs % 2 && c->opts.mem_budget == 0 ? 1 : 0); }
 static RhsLanes rhs_lanes(const aim_ctx* c, int B) {
   const int even = B + B % 2;
   const bool few = c->N < 152 * 8 * kNearGroup && B <= 32;
   RhsLanes r{};
-  r.rl = B > 16 && !few && even <= rhs_columns(c) ? 2 : 1;
+  r.rl = B > 16 && !few && even <= rhs_columns(c->max_rhs, c->opts.mem_budget) ? 2 : 1;
   r.lg = B <= 16 * r.rl && !few ? 16 : 32;
   r.ld = r.rl == 2 ? even : B;
   return r;
@@ -997,7 +996,7 @@ static int ensure_near_groups(aim_ctx* c, PrecData<R>& pd) {
 
 // RHS-minor copies of Phi and x for the many-RHS kernels (rhs_columns per row).
 template <typename R> static int ensure_rhs_minor(aim_ctx* c, PrecData<R>& pd) {
-  const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2], cols = rhs_columns(c);
+  const long long Nc = (long long)c->n[0] * c->n[1] * c->n[2], cols = rhs_columns(c->max_rhs, c->opts.mem_budget);
   if (pd.xT) return AIM_OK;
   const int rc = [&]() -> int {
     AIM_CUDA_TRY(cudaMalloc(&pd.phiT, sizeof(cplx<R>) * cols * 4 * Nc));
