@@ -4,12 +4,12 @@ Each request is one scatterer (mesh, wavenumber, excitation set) to be solved
 with FP64-refined complex64 AIM (``aim_solve`` with AIM_C64).  The server
 keeps ``slots`` worker threads, each with its own CUDA stream.  A request is
 admitted as soon as a slot is free and its estimated device footprint
-(``aim_footprint``) fits in the memory budget that the running requests have
-not claimed; admission is in arrival order, but a request that does not fit
-does not block later requests that do (up to ``max_skip`` passes).  Admitted
-requests run concurrently: their setup (host), spectra, products and Krylov
-steps interleave on the device.  The library calls release the GIL, so the
-threads overlap.
+(``aim_footprint``, and ``RCS_WORKSPACE`` if it asks for a pattern) fits in the
+memory budget that the running requests have not claimed; admission is in
+arrival order, but a request that does not fit does not block later requests
+that do (up to ``max_skip`` passes).  Admitted requests run concurrently: their
+setup (host), spectra, products and Krylov steps interleave on the device.  The
+library calls release the GIL, so the threads overlap.
 
 Two batching levels sit on top (``cache=True``, the default):
 
@@ -55,6 +55,10 @@ from . import (
     aim_setup,
     aim_solve,
 )
+
+
+# what a context may keep on the device after its first aim_rcs (aim.h), outside aim_footprint's estimate
+RCS_WORKSPACE = 64 << 20
 
 
 @dataclasses.dataclass
@@ -157,12 +161,12 @@ class Server:
         self.batches = []  # sizes of the solves run
 
     # -------------------------------------------------------------- admission
-    def _evict_idle(self, need):
-        """Free idle resident contexts, least recently used first, until `need` bytes fit (under the lock)."""
+    def _evict_idle(self, need, keep=None):
+        """Free idle resident contexts but `keep`, least recently used first, until `need` bytes fit (under the lock)."""
         for key, ent in sorted(self.contexts.items(), key=lambda kv: kv[1]["used"]):
             if self.claimed + need <= self.budget:
                 break
-            if ent["busy"]:
+            if ent["busy"] or ent is keep:
                 continue
             ent["ctx"].close()
             self.claimed -= ent["fp"]
@@ -171,34 +175,37 @@ class Server:
     def _admissible(self):
         """Pop the first pending request that can run now, with the pending requests
         that merge into its solve (under the lock).  Returns (batch, claim) or None;
-        claim is the footprint charged for the batch's duration (0 when it reuses a
-        resident context, whose footprint stays claimed while it is resident)."""
+        claim is the footprint charged for the batch's duration (when it reuses a
+        resident context, whose footprint stays claimed while it is resident, only
+        what the request needs beyond that: its pattern's workspace)."""
         for i, (req, fp, key) in enumerate(self.pending[: self.max_skip]):
             ent = self.contexts.get(key) if self.cache else None
             if ent is not None and ent["busy"]:
                 continue  # its context is solving: this request waits for it (or merges into the next solve)
-            need = 0 if ent is not None else fp
+            held = ent["fp"] if ent is not None else 0
+            need = max(0, fp - held)
             if self.cache and need and self.claimed + need > self.budget:
-                self._evict_idle(need)
-            if need == 0 or self.claimed + need <= self.budget or (self.busy == 0 and self.claimed == 0):
+                self._evict_idle(need, keep=ent)
+            if need == 0 or self.claimed + need <= self.budget or (self.busy == 0 and self.claimed == held):
                 self.pending.pop(i)
                 batch = [req]
                 if self.cache:
                     tot = len(req.khat)
                     j = 0
                     while j < len(self.pending):
-                        r2, _fp2, k2 = self.pending[j]
-                        if k2 == key and tot + len(r2.khat) <= self.merge_rhs:
+                        r2, fp2, k2 = self.pending[j]
+                        more = max(0, fp2 - held - need)
+                        if (k2 == key and tot + len(r2.khat) <= self.merge_rhs
+                                and (more == 0 or self.claimed + need + more <= self.budget)):
                             batch.append(r2)
                             tot += len(r2.khat)
+                            need += more
                             self.pending.pop(j)
                         else:
                             j += 1
                     if ent is None:  # the context this solve builds stays resident
-                        self.contexts[key] = {"ctx": None, "fp": fp, "busy": True, "used": time.perf_counter()}
-                    else:
-                        ent["busy"] = True
-                        ent["used"] = time.perf_counter()
+                        ent = self.contexts[key] = {"ctx": None}
+                    ent.update(fp=held + need, busy=True, used=time.perf_counter())
                     if self.pack > 1:
                         need += self._pack_more(req, key, batch, need)
                 return batch, need
@@ -219,7 +226,8 @@ class Server:
             v2 = box_volume(r2)
             fits = (k2 not in keys and pack_class(r2) == cls and max(v2, vol) <= self.pack_ratio * min(v2, vol)
                     and tot + len(r2.khat) <= self.pack_rhs and not (ent2 is not None and ent2["busy"]))
-            need2 = 0 if ent2 is not None else fp2
+            held2 = ent2["fp"] if ent2 is not None else 0
+            need2 = max(0, fp2 - held2)
             if not fits or (need2 and self.claimed + need + extra + need2 > self.budget):
                 j += 1
                 continue
@@ -228,10 +236,13 @@ class Server:
             ntot = len(r2.khat)
             i = j
             while i < len(self.pending):  # its own followers, as for the first scatterer
-                r3, _fp3, k3 = self.pending[i]
-                if k3 == k2 and ntot + len(r3.khat) <= self.merge_rhs and tot + ntot + len(r3.khat) <= self.pack_rhs:
+                r3, fp3, k3 = self.pending[i]
+                more = max(0, fp3 - held2 - need2)
+                if (k3 == k2 and ntot + len(r3.khat) <= self.merge_rhs and tot + ntot + len(r3.khat) <= self.pack_rhs
+                        and (more == 0 or self.claimed + need + extra + need2 + more <= self.budget)):
                     group.append(r3)
                     ntot += len(r3.khat)
+                    need2 += more
                     self.pending.pop(i)
                 else:
                     i += 1
@@ -240,10 +251,8 @@ class Server:
             keys.add(k2)
             extra += need2
             if ent2 is None:
-                self.contexts[k2] = {"ctx": None, "fp": fp2, "busy": True, "used": time.perf_counter()}
-            else:
-                ent2["busy"] = True
-                ent2["used"] = time.perf_counter()
+                ent2 = self.contexts[k2] = {"ctx": None}
+            ent2.update(fp=held2 + need2, busy=True, used=time.perf_counter())
         return extra
 
     def _make_stream(self):
@@ -419,8 +428,8 @@ class Server:
 
     def _footprint(self, req):
         nrhs = max(self.merge_rhs, len(req.khat)) if self.cache else len(req.khat)
-        return aim_footprint(req.verts, req.tris, req.h, req.M, req.near_radius, nrhs, req.cfie_alpha,
-                             self.precision)
+        fp = aim_footprint(req.verts, req.tris, req.h, req.M, req.near_radius, nrhs, req.cfie_alpha, self.precision)
+        return fp + (RCS_WORKSPACE if req.rcs_dirs is not None else 0)
 
     def close(self):
         """Free every resident context."""
