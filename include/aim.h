@@ -332,8 +332,9 @@ int aim_probe_fma_peak(int which, double* tflops);
  *   AIM_FFT_FOURSTEP        four-step register kernel (every padded length up to
  *                           900 and 1296; a longer one falls back to the
  *                           Stockham kernel);
- *   AIM_FFT_FOURSTEP_SMALL  four-step with blocks of at most 128 threads, one
- *                           pencil per thread (the x pass; elsewhere as
+ *   AIM_FFT_FOURSTEP_SMALL  four-step with blocks of at most 128 threads (the
+ *                           x pass of AIM_C128 and AIM_C128_F64; elsewhere, and
+ *                           for AIM_C64, whose blocks are that small, as
  *                           AIM_FFT_FOURSTEP);
  *   AIM_FFT_FOURSTEP_WARP, AIM_FFT_FOURSTEP_WIDE  accepted; run as
  *                           AIM_FFT_FOURSTEP.

@@ -79,8 +79,10 @@ static int autotune(aim_ctx* c, int precision, int nrhs, int reps, int32_t* kern
     const bool fourstep = fourstep_split(c->L[axis], &l1, &l2);  // else every choice runs Stockham
     double best_ms = 0.0;
     for (int k = AIM_FFT_STOCKHAM; k < AIM_FFT_KERNELS && rc == AIM_OK; ++k) {
-      // the x pass has a small-block variant; the warp-group and wide choices run the plain four-step kernel
-      if (k == AIM_FFT_FOURSTEP_WARP || k == AIM_FFT_FOURSTEP_WIDE || (k == AIM_FFT_FOURSTEP_SMALL && pass != 2)) continue;
+      // the x pass of the 16-byte types has a small-block variant (complex64 runs in such blocks anyway); the
+      // warp-group and wide choices run the plain four-step kernel
+      if (k == AIM_FFT_FOURSTEP_WARP || k == AIM_FFT_FOURSTEP_WIDE) continue;
+      if (k == AIM_FFT_FOURSTEP_SMALL && (pass != 2 || precision == AIM_C64)) continue;
       if (k != AIM_FFT_STOCKHAM && !fourstep) continue;
       c->fft_kernel[pol][pass] = k;
       double ms = 0.0;

@@ -13,7 +13,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from aim_inputs import random_complex  # noqa: E402
+from aim_inputs import plate_mesh, random_complex  # noqa: E402
 from oracle import aim as oaim  # noqa: E402
 from oracle.rwg import RWG  # noqa: E402
 from test_gpu_fft_lengths import H, K0, reachable, strip  # noqa: E402
@@ -95,4 +95,15 @@ def test_an_x_axis_without_a_four_step_kernel():
         assert np.linalg.norm(y.cpu().numpy() - ref) <= bound * np.linalg.norm(ref), prec
         kernels, ms = g.aim_autotune(ctx, prec, nrhs=2, reps=1)
         assert kernels[2] == g.AIM_FFT_STOCKHAM and ms[2, 1] > 0 and (ms[2, 2:] == -1).all()
+    ctx.close()
+
+def test_autotune_times_a_kernel_once():
+    """Small blocks are a kernel of their own in the 16-byte types only: complex64
+    x passes run in them anyway."""
+    ctx = g.aim_setup(*plate_mesh(1.0, 9), K0, H, M=2, max_rhs=1, planar=False)
+    for prec in BOUND:
+        kernels, ms = g.aim_autotune(ctx, prec, nrhs=1, reps=1)
+        tried = [1, 2] if prec == g.AIM_C64 else [1, 2, 3]
+        assert [k for k in range(g.AIM_FFT_KERNELS) if ms[2, k] > 0] == tried, prec
+        assert kernels[2] in tried
     ctx.close()
