@@ -311,21 +311,21 @@ struct LaunchScope {
     __VA_ARGS__;                          \
   } while (0)
 // The kernels of a small product are launched so that one may be set up while
-// the previous one still runs (programmatic stream serialisation): each first
-// allows its successor the same and then waits for its predecessor to be
-// complete and its writes visible, before it touches memory.  A kernel that is
-// not launched this way starts and ends as usual.  A 1 lambda plate's six
-// launches: 32.8 -> 22.4 us.  Not for kernels bound by the FP64 pipe (overlap =
-// false; the solver's launches are plain): blocks that start while others still
-// run land unevenly on the SMs, each of which has its own two FP64 lanes a
-// clock (a 4 lambda plate in native FP64: 77 -> 146 us).  Nor for a launch
-// larger than one wave, which gains nothing (32 lambda plate, 64 right-hand
-// sides: 1.70 -> 1.73 ms).
+// the previous one's last blocks run out (programmatic stream serialisation):
+// each waits for its predecessor to be complete and its writes visible before
+// it touches memory.  A kernel that is not launched this way starts and ends
+// as usual.  No kernel asks for its successor early (griddepcontrol.
+// launch_dependents): blocks placed while others still run land unevenly on the
+// SMs, and a launch takes as long as its fullest SM.  A 6 lambda plate, two
+// float-float right-hand sides, whose strided passes hold 32 SMs: 60 us without
+// overlap, 72 with early successors, 48 so; an 8 lambda plate, complex64, two:
+// 32, 29, 23; a 1.8 lambda sphere, complex64, one: 51, 53, 37.  Off for kernels
+// bound by the FP64 pipe (overlap = false; early successors took a 4 lambda
+// plate in native FP64 from 77 to 146 us, this form was not measured there), for
+// the solver's launches, and above 152 x 2048 threads, where the start of a
+// launch no longer counts.
 #ifdef __CUDACC__
-__device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... K, class... A>
 cudaError_t launch_pdl(bool overlap, void (*kernel)(K...), dim3 grid, dim3 block, size_t shared, cudaStream_t stream, A&&... args) {
   cudaLaunchAttribute attr[1];
