@@ -472,9 +472,12 @@ static_assert(kNearGroup == 4, "load_group reads four entries");
 // in shared memory and written back in the [B][N] layout.  Bound by the latency
 // of the runs' gathers, so complex64 keeps to 64 registers (80 with the MFIE
 // weights) for the warps' sake, with some values spilled (32 lambda plate, 64
-// right-hand sides: 911 us at 88 registers, 695 at 64).
-template <class MI, int RL, bool MF, int LG>
-__global__ void __launch_bounds__(256, sizeof(typename MI::R) > 4 ? 1 : MF ? 3 : 4) interp_near_grp(const cplx<typename MI::R>* __restrict__ PhiT,
+// right-hand sides: 911 us at 88 registers, 695 at 64).  CAP = false, where the
+// launch has no more blocks than are resident at the registers it asks for (108
+// and 128, two a SM; 136 and 165 with the MFIE weights, one): the product of a 1
+// lambda sphere with 64 right-hand sides takes 319 us without the spills, 351 with.
+template <class MI, int RL, bool MF, int LG, bool CAP>
+__global__ void __launch_bounds__(256, sizeof(typename MI::R) > 4 || !CAP ? 1 : MF ? 3 : 4) interp_near_grp(const cplx<typename MI::R>* __restrict__ PhiT,
                                                        const cplx<typename MI::R>* __restrict__ xT,
                                                        cplx<typename MI::R>* __restrict__ y,
                                                        const typename MI::R* __restrict__ lam,
@@ -1072,20 +1075,28 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
       with_lanes(rl, [&](auto l, auto w) {
         constexpr bool MF = decltype(mf)::value;
         constexpr int RL = decltype(l)::value, LG = decltype(w)::value, rows = 256 / LG * kNearGroup;
-        const auto kern = interp_near_grp<MI, RL, MF, LG>;
         const int blocks = (c->N + rows - 1) / rows;
         const size_t sm = sizeof(cplx<R>) * rows * (nrhs + 1);
-        // staged rows: at most 32 x 256 complex128 (128 KB), beside the stencil offsets
-        static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (attr != cudaSuccess) {
-          set_error(std::string("interp_near: ") + cudaGetErrorString(attr));
-          rc = AIM_ECUDA;
-          return;
-        }
-        AIM_LAUNCH(c, "interp_near",
-                   (launch_pdl(sizeof(typename MI::R) == 4, kern, blocks, 256, sm, c->stream, pd.phiT, pd.xT, y, lam,
-                               c->base, c->ngrp_ptr, c->ngrp_col, pd.ngrp_val, c->N, Nc, c->n[0], c->n[1], nrhs, rl.ld,
-                               fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
+        const auto run = [&](auto cap) {
+          const auto kern = interp_near_grp<MI, RL, MF, LG, decltype(cap)::value>;
+          // staged rows: at most 32 x 256 complex128 (128 KB), beside the stencil offsets
+          static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+          if (attr != cudaSuccess) {
+            set_error(std::string("interp_near: ") + cudaGetErrorString(attr));
+            rc = AIM_ECUDA;
+            return;
+          }
+          AIM_LAUNCH(c, "interp_near",
+                     (launch_pdl(sizeof(typename MI::R) == 4, kern, blocks, 256, sm, c->stream, pd.phiT, pd.xT, y, lam,
+                                 c->base, c->ngrp_ptr, c->ngrp_col, pd.ngrp_val, c->N, Nc, c->n[0], c->n[1], nrhs, rl.ld,
+                                 fvec, frho, c->S, c->M + 1, pd.lamM, fmf)));
+        };
+        // one wave: EFIE products of 188 to 240 blocks 5 to 9 % faster uncapped (spheres of 1.4 to 2
+        // lambda, 18 to 40 right-hand sides), of 345 to 454 blocks 2 to 3 % slower; CFIE ones of 120
+        // blocks 9 to 12 % faster, of 227 and 240 blocks 2 to 7 % slower
+        if constexpr (sizeof(R) == 4)
+          if (blocks > (MF ? 1 : 2) * 152) return run(std::true_type{});
+        run(std::false_type{});
       });
     };
     if (pd.lamM) go(std::true_type{}); else go(std::false_type{});
