@@ -93,13 +93,19 @@ struct ProjTasks {
 // start).  The next task's list bounds are loaded while the current one is
 // summed, and the right-hand sides go in chunks of BC: an entry's weights
 // and column are loaded once per chunk and its BC gathers of x are
-// independent loads.  U entries are in flight per lane, as many as leave the
-// registers for full residency (one right-hand side: 64 lambda plate, 51 us
-// with one entry, 45 with four; 10 lambda sphere, 97 us, 91).  Four right-hand
-// sides take two where the tasks are a single wave of blocks, which then only
-// wait for their loads (a 5 lambda plate: 10.9 -> 9.0 us), one beyond, where the
-// registers of a second cost resident warps (7 lambda sphere: 107 us, 127).
-constexpr int gather_unroll(int bc, bool one_wave) { return bc == 1 ? 4 : one_wave ? 2 : bc == 2 ? 4 : 1; }
+// independent loads.  U entries are in flight per lane.
+// Complex64: as many as leave the registers for full residency for one
+// right-hand side (64 lambda plate, 51 us with one entry, 45 with four; 10 lambda
+// sphere, 97 us, 91); where the tasks are a single wave of blocks, which then
+// only wait for their loads, four for two right-hand sides and two for four (a 5
+// lambda plate: 11.4 us with one, 12.4 with two, 10.8 with four; 10.9 -> 9.0 us);
+// one beyond, where the registers of a second cost resident warps (two, 7 lambda
+// sphere: 76 us with one, 87 with two, 84 with four; four: 107 us, 127).  Native
+// FP64 is bound by its pipe: one (3 lambda sphere, two right-hand sides: 98 us,
+// 111 with four).
+template <class R> constexpr int gather_unroll(int bc, bool one_wave) {
+  return sizeof(R) == 8 ? 1 : bc == 1 ? 4 : !one_wave ? 1 : bc == 2 ? 4 : 2;
+}
 template <class MD, int BC, int U>
 __global__ void __launch_bounds__(256) proj_gather(const cplx<typename MD::R>* __restrict__ x, typename MD::S* __restrict__ Q,
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ mm,
@@ -188,9 +194,10 @@ constexpr int kMaxStencil = 216;
 // right-hand sides: 1.82 -> 1.38 ms; 7 lambda sphere, CFIE, 4: 267 -> 206 us,
 // at 64 registers, for the warps' sake); a small body takes a whole warp per
 // basis function, which leaves one or two rounds of gathers where 8 lanes take
-// five to ten.
+// five to ten.  64 registers also for one FP64 right-hand side (32 lambda plate: 397 us, 428 at the
+// 105 it takes otherwise).
 template <class MD, bool MF, int BC, int W>
-__global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 ? 4 : 2) interp_near(const typename MD::S* __restrict__ Phi,
+__global__ void __launch_bounds__(256, sizeof(typename MD::R) == 4 || (BC == 1 && !MF) ? 4 : 2) interp_near(const typename MD::S* __restrict__ Phi,
                                                    const cplx<typename MD::R>* __restrict__ x,
                                                    cplx<typename MD::R>* __restrict__ y,
                                                    const typename MD::R* __restrict__ lam,
@@ -1053,10 +1060,10 @@ static int run_product(aim_ctx* c, const cplx<typename MD::R>* x, cplx<typename 
     const auto go = [&](auto bc) {
       constexpr int BC = decltype(bc)::value;
       if (blocks <= 2 * 152)
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll(BC, true)>, blocks, 256, 0, c->stream, 
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll<R>(BC, true)>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
       else
-        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll(BC, false)>, blocks, 256, 0, c->stream, 
+        AIM_LAUNCH(c, "proj_gather", (launch_pdl(sizeof(typename MD::R) == 4, proj_gather<MD, BC, gather_unroll<R>(BC, false)>, blocks, 256, 0, c->stream, 
                                          x, grid0, c->pnode_ptr, c->pnode_m, pw, c->N, Nc, nrhs, groups, ntask)));
     };
     if (nrhs == 1) go(std::integral_constant<int, 1>{});
@@ -1215,7 +1222,7 @@ int matvec_c64_bufs(aim_ctx* c, const float2* x, float2* y, int nrhs, float2* g0
     const int blocks = (int)std::min<long long>((ntask + 7) / 8, 152LL * 16);
     const auto go = [&](auto bc) {
       constexpr int BC = decltype(bc)::value;
-      AIM_LAUNCH(c, "proj_gather", (launch_pdl(true, proj_gather<M32, BC, gather_unroll(BC, false)>, blocks, 256, 0, c->stream, 
+      AIM_LAUNCH(c, "proj_gather", (launch_pdl(true, proj_gather<M32, BC, gather_unroll<float>(BC, false)>, blocks, 256, 0, c->stream, 
                                        x, g0, c->pnode_ptr, c->pnode_m, c->p32.pnode_w, c->N, Nc, nrhs, nullptr,
                                        ntask)));
     };
