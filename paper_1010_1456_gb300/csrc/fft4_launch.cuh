@@ -94,8 +94,35 @@ int launch_x4(aim_ctx* c, const char* name, S* buf, XArgs4 a, const S* ghat, con
     const int split = (int)std::min<long long>(rounds, (12LL * kSMs + rows() - 1) / rows());
     GB = (rounds + split - 1) / split * TG;
   }
-  while (more() && RY > 1) RY = (RY + 1) / 2;
-  while (more() && TG > 1) GB = TG = (TG + 1) / 2;
+  if (std::is_same<Pol, P64>::value) {
+    // Bound by the FP64 pipe, where a warp costs the same with any number of its lanes in use: the smallest
+    // blocks, as below, unless another of these shapes leaves the busiest SM a tenth less warp time (324 x
+    // 324 plane, 4 grids: 648 blocks of 36 units, 105 us; 108 blocks of 216, 72; 400: 128 and 88)
+    struct Shape {
+      int ry, tg, gb;
+      double t;
+    };
+    const auto shape = [&] {
+      const int n = RY * TG;
+      const double AC = 2.0 * ((n * L2 + 31) / 32) * L1 * std::log2(L1 + 1.0),
+                   B = (double)((n * L1 + 31) / 32) * (2 * L2 * std::log2(L2 + 1.0) + L2);
+      return Shape{RY, TG, GB, (AC + B) * ((GB + TG - 1) / TG) * (double)((blocks() + kSMs - 1) / kSMs)};
+    };
+    Shape best = shape(), last = best;
+    while (more() && (RY > 1 || TG > 1)) {
+      if (RY > 1) RY = (RY + 1) / 2;
+      else GB = TG = (TG + 1) / 2;
+      last = shape();
+      if (last.t < best.t) best = last;
+    }
+    if (best.t >= 0.9 * last.t) best = last;
+    RY = best.ry;
+    TG = best.tg;
+    GB = best.gb;
+  } else {
+    while (more() && RY > 1) RY = (RY + 1) / 2;
+    while (more() && TG > 1) GB = TG = (TG + 1) / 2;
+  }
   a.RY = RY;
   a.TG = TG;
   a.GB = GB;

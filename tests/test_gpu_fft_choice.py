@@ -62,6 +62,21 @@ def test_an_explicit_four_step_x_pass_runs(L):
     ctx.close()
 
 
+@pytest.mark.parametrize("side, L", [(0.9, 24), (3.2, 72), (6.5, 135), (16.0, 324), (19.2, 400)])
+def test_x_pass_shapes_on_a_plane(side, L):
+    """Planar grids of 1 to 5 right-hand sides: few rows, which the x pass lays over
+    blocks by the number of grids, down to one row and one grid a block."""
+    ctx = g.aim_setup(*plate_mesh(side, int(round(9 * side))), K0, H, M=2, max_rhs=5)
+    assert g.aim_grid_info(ctx)[1] == [L, L, 1]
+    x = torch.from_numpy(random_complex((5, ctx.N), L)).cuda()
+    for nrhs in (1, 2, 5):
+        xs = x[:nrhs].contiguous()
+        for prec, bound in BOUND.items():
+            ref = product(ctx, xs, prec, g.AIM_FFT_STOCKHAM)
+            assert rel(product(ctx, xs, prec, g.AIM_FFT_FOURSTEP), ref) <= 2 * bound, (nrhs, prec)
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec", [g.AIM_C128, g.AIM_C128_F64])
 def test_the_rule_on_both_sides_of_its_line(prec):
     """125 = 5 x 25 points, 8 x 5 rows: 1,000 units a grid, 4 grids a right-hand
