@@ -324,10 +324,11 @@ int aim_probe_fma_peak(int which, double* tflops);
  * forward transform, spectral product, inverse -- y inverse, z inverse, in
  * that order) runs one of:
  *   AIM_FFT_AUTO            the built-in rule (default): four-step where the padded
- *                           length has such a kernel, except Stockham for x passes
- *                           of AIM_C128 and AIM_C128_F64 with few pencils and
- *                           register DFTs of 24 points or more (padded x lengths
- *                           125, 243, 250, 375 and from 384 on all but 400);
+ *                           length has such a kernel, except Stockham for passes
+ *                           of AIM_C128 and AIM_C128_F64 over few pencils with long
+ *                           register DFTs (the x pass of padded lengths 125, 243,
+ *                           250, 375 and from 384 on all but 400; the other
+ *                           passes of 125);
  *   AIM_FFT_STOCKHAM        mixed-radix Stockham kernel (any 2,3,5-smooth length);
  *   AIM_FFT_FOURSTEP        four-step register kernel (every padded length up to
  *                           900 and 1296; a longer one falls back to the

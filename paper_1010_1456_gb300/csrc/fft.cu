@@ -377,11 +377,16 @@ bool fourstep_split(int L, int* L1, int* L2) {
 int fft_policy_of(int precision) { return precision == AIM_C64 ? 0 : precision == AIM_C128_F64 ? 1 : 2; }
 
 // AIM_FFT_AUTO is the four-step kernel where the padded length has one, but for a few float-float or
-// FP64 pencils with long register DFTs in the x pass: too few units to hide their serial chains, and the
-// Stockham kernel's radix-5 and smaller steps use more threads (375 x 375 plane, 4 float-float grids: 54 us
-// four-step, 33 Stockham; 432: 35 and 33; FP64 135 and 107).  From 58 k units on the four-step kernel is the
-// faster one (648 x 648, 8 grids, 140 k units: 122 us, 164), and with DFTs of at most 20 it always was (320
-// plane, FP64: 70 and 77).
+// FP64 pencils with long register DFTs: too few units to hide their serial chains, and the Stockham
+// kernel's radix-5 and smaller steps use more threads.  In the x pass DFTs of 24 and more give way below
+// 58 k units (a plane of one right-hand side, us four-step / Stockham: float-float 375 x 375, 37 k, 54 / 33,
+// 432 35 / 33; FP64 125, 12 k, 45 / 23), with DFTs of at most 20 they do not (320 plane, FP64: 70 / 77), nor
+// above (648, 70 k: float-float 87 / 87, FP64 258 / 303).  The DFT of 25 has no prime-factor split and gives
+// way below 66 k (FP64 625, 62 k: 378 / 332), and in float-float, where it spills at the x pass's registers,
+// below 304 k (625 with four right-hand sides, 250 k: 296 / 285; 500, 200 k: 217 / 178; 125 with eight, 100 k,
+// and 450 with four, 180 k, are level and 13 % better four-step; 125 x 125 x 125, 1.6 M: 236 / 273).
+// The strided passes follow the x pass's line where the split is as uneven as 125's, whose 5-point step
+// leaves four threads in five idle (FP64 plane: 25 / 18; 125 x 125 x 125, 790 k units: 237 / 271).
 int fft_kernel_for(const aim_ctx* c, int pol, int pass, int G) {
   const int k = c->fft_kernel[pol][pass];
   if (k != AIM_FFT_AUTO) return k;
@@ -389,8 +394,11 @@ int fft_kernel_for(const aim_ctx* c, int pol, int pass, int G) {
   if (c->L[axis] == 1) return AIM_FFT_FOURSTEP;  // a planar grid's z passes, which do not run
   int l1 = 0, l2 = 0;
   if (!fourstep_split(c->L[axis], &l1, &l2)) return AIM_FFT_STOCKHAM;
-  const long long units = (long long)G * c->L[1] * c->L[2] * std::max(l1, l2);
-  return pass == 2 && pol != 0 && std::max(l1, l2) >= 24 && units < 384LL * 152 ? AIM_FFT_STOCKHAM : AIM_FFT_FOURSTEP;
+  const int lm = std::max(l1, l2), ls = std::min(l1, l2);
+  if (pol == 0 || lm < 24 || (pass != 2 && lm < 5 * ls)) return AIM_FFT_FOURSTEP;
+  const long long pencils = axis == 0 ? (long long)c->L[1] * c->L[2] : (long long)c->n[0] * (axis == 1 ? c->L[2] : c->n[1]);
+  const long long line = lm != 25 ? 384 : pass == 2 && pol == 2 ? 2000 : 432;
+  return G * pencils * lm < line * 152 ? AIM_FFT_STOCKHAM : AIM_FFT_FOURSTEP;
 }
 
 template <class P> constexpr int policy_index() {

@@ -77,18 +77,37 @@ def test_x_pass_shapes_on_a_plane(side, L):
     ctx.close()
 
 
-@pytest.mark.parametrize("prec", [g.AIM_C128, g.AIM_C128_F64])
-def test_the_rule_on_both_sides_of_its_line(prec):
+@pytest.mark.parametrize("prec, nrhs", [(g.AIM_C128, 76), (g.AIM_C128_F64, 17)])
+def test_the_rule_on_both_sides_of_its_line(prec, nrhs):
     """125 = 5 x 25 points, 8 x 5 rows: 1,000 units a grid, 4 grids a right-hand
-    side; the line is at 58,368 units, between 14 and 15 right-hand sides."""
+    side; the line is at 304,000 units (float-float DFTs of 25) and 65,664 (FP64)."""
     v, t = strip(125, 0, wide=False)
-    ctx = g.aim_setup(v, t, K0, H, M=2, max_rhs=15)
+    ctx = g.aim_setup(v, t, K0, H, M=2, max_rhs=nrhs)
     assert g.aim_grid_info(ctx)[1] == [125, 8, 5]
     assert g.aim_fft_config(ctx, prec)[2] == g.AIM_FFT_FOURSTEP  # resolved for max_rhs
-    x = torch.from_numpy(random_complex((15, ctx.N), 3)).cuda()
-    for nrhs, k in ((15, g.AIM_FFT_FOURSTEP), (14, g.AIM_FFT_STOCKHAM)):
-        xs = x[:nrhs].contiguous()
-        assert torch.equal(product(ctx, xs, prec, g.AIM_FFT_AUTO), product(ctx, xs, prec, k)), nrhs
+    x = torch.from_numpy(random_complex((nrhs, ctx.N), 3)).cuda()
+    for n, k in ((nrhs, g.AIM_FFT_FOURSTEP), (nrhs - 1, g.AIM_FFT_STOCKHAM)):
+        xs = x[:n].contiguous()
+        assert torch.equal(product(ctx, xs, prec, g.AIM_FFT_AUTO), product(ctx, xs, prec, k)), n
+    ctx.close()
+
+
+@pytest.mark.parametrize("along, passes", [(1, (1, 3)), (2, (0, 4))])
+def test_the_rule_of_the_strided_passes(along, passes):
+    """125 points along y or z of a strip: Stockham in the 16-byte types' passes of
+    that axis, four-step in complex64's, and what is reported is what runs."""
+    ctx = g.aim_setup(*strip(125, along, wide=False), K0, H, M=2, max_rhs=2)
+    assert g.aim_grid_info(ctx)[1][along] == 125
+    x = torch.from_numpy(random_complex((2, ctx.N), 4)).cuda()
+    for prec in BOUND:
+        xp = x.to(torch.complex64) if prec == g.AIM_C64 else x
+        y = g.aim_matvec(ctx, xp, precision=prec)
+        ran = g.aim_fft_config(ctx, prec)
+        assert ran == [1 if prec != g.AIM_C64 and p in passes else 2 for p in range(5)]
+        g.aim_fft_config(ctx, prec, ran)
+        assert torch.equal(y, g.aim_matvec(ctx, xp, precision=prec))
+        g.aim_fft_config(ctx, prec, [g.AIM_FFT_FOURSTEP] * 5)
+        assert rel(g.aim_matvec(ctx, xp, precision=prec), y) <= 2 * BOUND[prec]
     ctx.close()
 
 
