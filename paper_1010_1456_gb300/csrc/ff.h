@@ -35,49 +35,12 @@ __device__ __forceinline__ ff ff_fast_two_sum(float a, float b) {
   return ff{s, e};
 }
 
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-  const ff s = ff_two_sum(a.hi, b.hi);
-  const float e = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-  return ff_fast_two_sum(s.hi, e);
-}
-
-// Addition without the closing renormalisation: hi is the rounded sum of the
-// high parts and lo collects that rounding error plus both low parts, so
-// hi + lo still carries the sum to about 2^-47 (|a| + |b|) but |lo| may
-// exceed ulp(hi)/2 by a few units.  Later TwoSum/TwoProduct steps accept
-// such pairs; used inside FFT butterflies, where every value feeds further
-// arithmetic.
-__device__ __forceinline__ ff ff_add_lazy(ff a, ff b) {
-  const ff s = ff_two_sum(a.hi, b.hi);
-  return ff{s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
-}
-
-__device__ __forceinline__ ff ff_neg(ff a) { return ff{-a.hi, -a.lo}; }
-__device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, ff_neg(b)); }
-
 __device__ __forceinline__ ff ff_mul(ff a, ff b) {
   const float p = __fmul_rn(a.hi, b.hi);
   float e = __fmaf_rn(a.hi, b.hi, -p);
   e = __fmaf_rn(a.hi, b.lo, e);
   e = __fmaf_rn(a.lo, b.hi, e);
   return ff_fast_two_sum(p, e);
-}
-
-// a * b - c * d and a * d + b * c style fused forms: one renormalisation for
-// the sum of two products (used by the complex product).
-__device__ __forceinline__ ff ff_dot2(ff a, ff b, ff c, ff d) {
-  // a*b + c*d
-  const float p1 = __fmul_rn(a.hi, b.hi);
-  const float p2 = __fmul_rn(c.hi, d.hi);
-  const ff s = ff_two_sum(p1, p2);
-  float e = __fmaf_rn(a.hi, b.hi, -p1);
-  e = __fadd_rn(e, __fmaf_rn(c.hi, d.hi, -p2));
-  e = __fmaf_rn(a.hi, b.lo, e);
-  e = __fmaf_rn(a.lo, b.hi, e);
-  e = __fmaf_rn(c.hi, d.lo, e);
-  e = __fmaf_rn(c.lo, d.hi, e);
-  e = __fadd_rn(e, s.lo);
-  return ff_fast_two_sum(s.hi, e);
 }
 
 // acc + a * b with one closing renormalisation: the product's rounding
@@ -98,7 +61,6 @@ __device__ __forceinline__ ff ff_from_double(double v) {
   const float lo = __double2float_rn(v - (double)hi);
   return ff{hi, lo};
 }
-__device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 
 // ------------------------------------------------------------------ two parts at a time
 // Two FP32 operations in one instruction (f32x2, each half rounded to
@@ -135,7 +97,12 @@ __device__ __forceinline__ cff2 fast_two_sum2(float2 a, float2 b) {
   const float2 s = add2(a, b);
   return cff2{s, sub2(b, sub2(s, a))};
 }
-// ff_add, ff_add_lazy, ff_dot2 and ff_mad of each part
+// Sums, sums of two products and ff_mad of each part.  The lazy sum leaves out
+// the closing renormalisation: hi is the rounded sum of the high parts and lo
+// collects that rounding error plus both low parts, so hi + lo still carries the
+// sum to about 2^-47 (|a| + |b|) but |lo| may exceed ulp(hi)/2 by a few units.
+// Later TwoSum/TwoProduct steps accept such pairs; used inside FFT butterflies,
+// where every value feeds further arithmetic.
 __device__ __forceinline__ cff2 cff2_add(cff2 a, cff2 b) {
   const cff2 s = two_sum2(a.hi, b.hi);
   return fast_two_sum2(s.hi, add2(s.lo, add2(a.lo, b.lo)));

@@ -137,15 +137,16 @@ __global__ void __launch_bounds__(256) proj_pack(const float2* __restrict__ x, f
 
 // Interpolation + near correction, W lanes per basis function of any instance
 // (they share one instance; the groups of a warp may not, so the reductions
-// use the group's own lane mask), BC right-hand sides at a time (as
+// use the group's own lane mask), four right-hand sides at a time (as
 // interp_near), then the padding of every packed row written as zero.
-template <int BC, int W>
+template <int W>
 __global__ void __launch_bounds__(256) interp_pack(const float2* __restrict__ Phi, const float2* __restrict__ x,
                                                    float2* __restrict__ y, const PackInst* __restrict__ inst,
                                                    const int32_t* __restrict__ row0, int K, long long rows, int ldx,
                                                    int nxp, int nyp, long long Ncp, int S, int P,
                                                    const int32_t* __restrict__ rhsN, int B) {
   pdl_begin();
+  constexpr int BC = 4;
   __shared__ int s_off[kPackMaxStencil];
   for (int s = threadIdx.x; s < S; s += blockDim.x) {
     const int ii = s % P, j = (s / P) % P, kk = s / (P * P);
@@ -259,12 +260,12 @@ static int pack_c64(aim_pack* P, const float2* x, float2* y) {
   }
   AIM_TRY(fft_convolve_c64(c, 4 * P->B));
   {
-    // a warp per basis function while 8 lanes would leave three quarters of the GPU's threads unused
+    // a warp per basis function while 8 lanes would leave seven eighths of the GPU's threads unused
     const auto go = [&](auto w) {
       constexpr int W = decltype(w)::value;
       const unsigned blocks = (unsigned)std::max<long long>(1, (P->rows * W + 255) / 256);
       AIM_LAUNCH(c, "interp_pack",
-                 (launch_pdl(true, interp_pack<4, W>, blocks, 256, 0, c->stream, phi_grid(c, c->p32.grid0, c->p32.grid2), x, y,
+                 (launch_pdl(true, interp_pack<W>, blocks, 256, 0, c->stream, phi_grid(c, c->p32.grid0, c->p32.grid2), x, y,
                                                                    P->d_inst, P->d_row0, P->K, P->rows, P->ld, c->n[0],
                                                                    c->n[1], Ncp, c->S, c->M + 1, P->d_rhsN, P->B)));
     };
