@@ -209,6 +209,11 @@ int aim_matvec_host(aim_ctx* ctx, const void* x_host, void* y_host, int nrhs, in
  * overwritten (initial guess 0).  info may be NULL.  Synchronises.  A
  * right-hand side holding NaN or an infinity is rejected with AIM_EINVAL
  * before any iteration (its norm, computed first, is not finite).
+ * Threads: contexts may be built, used and freed in other threads meanwhile
+ * (one context in one thread at a time).  The step's graph is captured from a
+ * stream of the library, and CUDA forbids a wait for the whole device
+ * (cudaDeviceSynchronize) while any stream captures: a program that solves in
+ * one thread waits for streams or events in the others.
  */
 int aim_solve(aim_ctx* ctx, const void* V_dev, void* X_dev, int nrhs, double tol, aim_solve_info* info);
 

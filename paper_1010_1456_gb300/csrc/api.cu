@@ -32,7 +32,7 @@ template <typename R> static void free_prec(PrecData<R>& p) {
 
 void free_context(aim_ctx* c) {
   if (!c) return;
-  cudaDeviceSynchronize();
+  device_wait();
   free_prec(c->p64);
   free_prec(c->p32);
   cudaFree(c->pff.ghat);

@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -388,6 +389,14 @@ int solve(aim_ctx* c, const double2* V, double2* X, int nrhs, double tol, aim_so
 // once, for aim_export.
 int fetch_host_arrays(aim_ctx* c);
 int alloc_krylov(aim_ctx* c);
+// Held while a step is captured and while the library waits for the whole device: that wait fails while
+// any stream captures, and spoils the capture.
+std::mutex& capture_mutex();
+inline void device_wait() {
+  std::lock_guard<std::mutex> lock(capture_mutex());
+  cudaDeviceSynchronize();
+  cudaGetLastError();  // refused while the program itself captures: not this thread's next launch's error
+}
 // api.cu: footprint estimate (aim_footprint), and the mem_budget check of the
 // grids of a product precision the setup's estimate did not count.
 int footprint_estimate(const aim_mesh* mesh, double h, int M, double near_radius, int max_rhs, double alpha,

@@ -399,6 +399,48 @@ void free_krylov(aim_ctx* c) {
   k = KrylovWork{};
 }
 
+std::mutex& capture_mutex() {
+  static std::mutex m;
+  return m;
+}
+
+// Runs the step that `body` launches, replayed from a CUDA graph that is captured on first use for this
+// key and batch size.  body(stream) launches everything on that stream.
+template <class F> static int replay_step(aim_ctx* c, int key, int nrhs, const char* what, F&& body) {
+  KrylovWork& k = c->kw;
+  const cudaStream_t st = c->stream;
+  if (!k.step_exec || k.step_prec != key || k.step_nrhs != nrhs) {
+    drop_step_graph(c);
+    const int64_t l0 = c->launches;
+    cudaGraph_t graph = nullptr;
+    int rc;
+    cudaError_t e;
+    {
+      std::lock_guard<std::mutex> lock(capture_mutex());
+      AIM_CUDA_TRY(cudaStreamBeginCapture(k.cap_stream, cudaStreamCaptureModeThreadLocal));
+      c->stream = k.cap_stream;  // every launch of the step goes to the capturing stream
+      rc = body(k.cap_stream);
+      c->stream = st;
+      e = cudaStreamEndCapture(k.cap_stream, &graph);
+    }
+    k.step_launches = c->launches - l0;
+    c->launches = l0;
+    if (rc == AIM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&k.step_exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (rc != AIM_OK) return rc;
+    if (e != cudaSuccess) {
+      k.step_exec = nullptr;
+      set_error(std::string("aim_solve: graph of the ") + what + ": " + cudaGetErrorString(e));
+      return AIM_ECUDA;
+    }
+    k.step_prec = key;
+    k.step_nrhs = nrhs;
+  }
+  c->launches += k.step_launches;
+  AIM_CUDA_TRY(cudaGraphLaunch(k.step_exec, st));
+  return AIM_OK;
+}
+
 // All of the solver's storage or none of it.
 int alloc_krylov(aim_ctx* c) {
   const int rc = fill_krylov(c);
@@ -484,42 +526,13 @@ struct Solver {
     allow_graph = false;  // the check build reads its index checks (a synchronisation) after every product
 #endif
     if (!allow_graph || c->prof.on) return step(precision);
-    if (!k.step_exec || k.step_prec != precision || k.step_nrhs != B) {
-      if (k.step_exec) {
-        cudaGraphExecDestroy(k.step_exec);
-        k.step_exec = nullptr;
-      }
-      const int64_t l0 = c->launches;
+    return replay_step(c, precision, B, "Arnoldi step", [&](cudaStream_t s) {
       const cudaStream_t st0 = st;
-      AIM_CUDA_TRY(cudaStreamBeginCapture(k.cap_stream, cudaStreamCaptureModeThreadLocal));
-      c->stream = st = k.cap_stream;  // every launch of the step goes to the capturing stream
+      st = s;
       const int rc = step(precision);
-      c->stream = st = st0;
-      cudaGraph_t graph = nullptr;
-      const cudaError_t e = cudaStreamEndCapture(k.cap_stream, &graph);
-      k.step_launches = c->launches - l0;
-      c->launches = l0;
-      if (rc != AIM_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc;
-      }
-      if (e != cudaSuccess) {
-        set_error(std::string("aim_solve: stream capture of the Arnoldi step: ") + cudaGetErrorString(e));
-        return AIM_ECUDA;
-      }
-      const cudaError_t ei = cudaGraphInstantiate(&k.step_exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (ei != cudaSuccess) {
-        k.step_exec = nullptr;
-        set_error(std::string("aim_solve: graph instantiation: ") + cudaGetErrorString(ei));
-        return AIM_ECUDA;
-      }
-      k.step_prec = precision;
-      k.step_nrhs = B;
-    }
-    c->launches += k.step_launches;
-    AIM_CUDA_TRY(cudaGraphLaunch(k.step_exec, st));
-    return AIM_OK;
+      st = st0;
+      return rc;
+    });
   }
 };
 }  // namespace
@@ -1046,43 +1059,7 @@ struct Tfqmr {
     allow_graph = false;  // the check build synchronises after every product
 #endif
     if (!allow_graph || c->prof.on) return pair(precision);
-    const int key = precision + 16;
-    if (!k.step_exec || k.step_prec != key || k.step_nrhs != B) {
-      if (k.step_exec) {
-        cudaGraphExecDestroy(k.step_exec);
-        k.step_exec = nullptr;
-      }
-      const int64_t l0 = c->launches;
-      const cudaStream_t st0 = c->stream;
-      AIM_CUDA_TRY(cudaStreamBeginCapture(k.cap_stream, cudaStreamCaptureModeThreadLocal));
-      c->stream = k.cap_stream;
-      const int rc = pair(precision);
-      c->stream = st0;
-      cudaGraph_t graph = nullptr;
-      const cudaError_t e = cudaStreamEndCapture(k.cap_stream, &graph);
-      k.step_launches = c->launches - l0;
-      c->launches = l0;
-      if (rc != AIM_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc;
-      }
-      if (e != cudaSuccess) {
-        set_error(std::string("aim_solve: stream capture of the TFQMR step: ") + cudaGetErrorString(e));
-        return AIM_ECUDA;
-      }
-      const cudaError_t ei = cudaGraphInstantiate(&k.step_exec, graph, 0);
-      cudaGraphDestroy(graph);
-      if (ei != cudaSuccess) {
-        k.step_exec = nullptr;
-        set_error(std::string("aim_solve: graph instantiation: ") + cudaGetErrorString(ei));
-        return AIM_ECUDA;
-      }
-      k.step_prec = key;
-      k.step_nrhs = B;
-    }
-    c->launches += k.step_launches;
-    AIM_CUDA_TRY(cudaGraphLaunch(k.step_exec, c->stream));
-    return AIM_OK;
+    return replay_step(c, precision + 16, B, "TFQMR step", [&](cudaStream_t) { return pair(precision); });
   }
 };
 }  // namespace

@@ -327,7 +327,7 @@ int pack_prepare(aim_ctx* c, int precision) {
 
 static void free_pack(aim_pack* P) {
   if (!P) return;
-  cudaDeviceSynchronize();
+  device_wait();
   cudaFree(P->d_inst);
   cudaFree(P->d_row0);
   cudaFree(P->d_rhsN);
